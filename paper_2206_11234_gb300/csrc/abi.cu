@@ -204,7 +204,6 @@ int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetCo
     std::memset(&c, 0, sizeof(c));
     c.phi_in = s.phi_in;
     c.phi_end = s.phi_end;
-    c.phi_uv = s.phi_uv;
     c.twouv = 2.0 * s.phi_uv;
     c.dN = s.dN;
     c.sq = std::sqrt(s.dN);
@@ -214,6 +213,7 @@ int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetCo
     c.lw_bsq = s.b * c.sq;
     c.lw_half_b2dN = 0.5 * s.b * s.b * s.dN;
     c.first = first;
+    c.ticket0 = first;
     c.traj_offset = s.traj_offset;
     c.m_max = (int)steps;
     c.set_id = s.set_id;
@@ -264,6 +264,80 @@ int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetCo
     return FPT_OK;
 }
 
+// Expected length of a run of the set and its spread, in steps: the noise-free
+// duration, the integral of dphi / |D + B|, and the small-noise standard
+// deviation, the square root of the integral of S^2 / |D + B|^3 dphi, by the
+// midpoint rule; at most the censoring cap, which is also taken (with no spread)
+// where the biased drift does not point down.
+static void expected_length(const fpt_params* p, const SetConst& c, double* steps, double* spread) {
+    constexpr int kNodes = 16;
+    *steps = *spread = 0.0;
+    if (!(c.phi_in > c.phi_end)) return;
+    const double h = (c.phi_in - c.phi_end) / kNodes;
+    double dur = 0.0, var = 0.0;
+    for (int i = 0; i < kNodes; ++i) {
+        const double x = c.phi_end + (i + 0.5) * h;
+        double D, S;
+        if (p->model == FPT_MODEL_CONSTANT) {
+            D = c.a0;
+            S = c.cm;
+        } else if (p->model == FPT_MODEL_POLYNOMIAL) {
+            double V = 0.0, dV = 0.0;
+            for (int k = FPT_POLY_TERMS - 1; k >= 0; --k) {
+                dV = dV * x + V;
+                V = V * x + c.poly[k];
+            }
+            D = -dV / V;
+            S = std::sqrt(V) / (2.0 * 3.14159265358979323846 * std::sqrt(3.0));
+        } else {
+            D = -2.0 / x;
+            S = c.cm * x;
+        }
+        const double v = -(D + (p->bias_kind == FPT_BIAS_POWER ? c.b * std::pow(x, c.pw) : c.b * S));
+        if (!(v > 0.0)) {
+            *steps = (double)c.m_max;
+            return;
+        }
+        dur += h / v;
+        var += h * S * S / (v * v * v);
+    }
+    *steps = std::fmin(dur / c.dN, (double)c.m_max);
+    *spread = std::sqrt(var) / c.dN;
+}
+
+void order_tickets(const fpt_params* p, SetConst* table, const fpt_set* sets, int n_sets, RunLengths* len) {
+    struct Item {
+        double steps, spread;
+        long long n;
+        int set;
+    };
+    std::vector<Item> order(n_sets);
+    *len = RunLengths{0.0, 0.0, 0.0};
+    for (int i = 0; i < n_sets; ++i) {
+        order[i].n = (long long)sets[i].n_traj;
+        order[i].set = i;
+        expected_length(p, table[i], &order[i].steps, &order[i].spread);
+        len->total += order[i].steps * (double)order[i].n;
+        if (order[i].n > 0) len->longest = std::fmax(len->longest, order[i].steps);
+    }
+    std::stable_sort(order.begin(), order.end(), [](const Item& a, const Item& b) { return a.steps > b.steps; });
+    // the tickets handed out last decide how long the launch trails off
+    long long last = 0;
+    for (int i = n_sets - 1; i >= 0 && last < kTrailingRuns; --i) {
+        last += order[i].n;
+        const double room = (double)table[order[i].set].m_max - order[i].steps;
+        if (order[i].n > 0) len->tail = std::fmax(len->tail, std::fmin(4.0 * order[i].spread, room));
+    }
+    if (n_sets < 2) return;
+    const std::vector<SetConst> from(table, table + n_sets);
+    long long ticket = 0;
+    for (int i = 0; i < n_sets; ++i) {
+        table[i] = from[order[i].set];
+        table[i].ticket0 = ticket;
+        ticket += order[i].n;
+    }
+}
+
 int check_hist(int32_t n_bins, double lo, double hi, int32_t n_sub) {
     if (n_bins < 1 || n_sub < 1) return fail(FPT_EINVAL, "n_bins %d and n_sub %d must be >= 1", n_bins, n_sub);
     if ((long long)n_bins * n_sub > FPT_MAX_HIST_BINS)
@@ -308,6 +382,7 @@ int prepare(const fpt_params* p, const fpt_set* sets, int n_sets, bool with_hist
         }
         P->n_total += (unsigned long long)sets[i].n_traj;
     }
+    order_tickets(p, P->sets.data(), sets, n_sets, &P->len);
     return FPT_OK;
 }
 
@@ -315,7 +390,6 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
     int b = p->block_dim;
     int s = p->k_steps;
     if (p->bias_kind == FPT_BIAS_POWER) {
-        if (b == 0) b = 256;
         if (p->precision == FPT_PREC_F64) {
             *k = stepper_f64(kModelPowReal, wall, s == 0 ? 4 : s);
         } else {
@@ -332,7 +406,6 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
             if (s == 0) s = ts;
         }
     }
-    if (b == 0) b = 256;
     if (p->precision == FPT_PREC_F64) {
         if (s == 0) s = 4;
         *k = stepper_f64(p->model, wall, s);
@@ -345,20 +418,61 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
     return FPT_OK;
 }
 
-int stepper_grid(const StepperKernel& k, int block, int n_sets, unsigned long long n_total, int* grid) {
+// The grid of the persistent stepper: as many warps per SM as fit, fewer where
+// the launch would trail off.  A run's speed is inversely proportional to the
+// warps that share its SM, the SM's throughput hardly depends on them (16 warps
+// per SM run 2.5 % slower than 32 on the drift ladder, 24 warps 1 %), so the last
+// and longest runs finish sooner with fewer.  In units of an SM's time per
+// warp-step, a full SM of r warps needs r x steps for one run's steps, and
+// total / (32 n_sm) for its share of the whole work; measured (us):
+//   tail / work                    16 warps   24 warps   32 warps
+//   0.7   3 x 50,000 diffusive runs   2809       3263       4075
+//   0.18  3 x 200,000                 8060       8040       8288
+//   0.09  3 x 400,000                15198      14884      15000
+//   0     3 x 65,536 capped runs     21859      21149      21097
+// The longest expected run bounds the launch as well (64 uneven sets of 4096:
+// 8020 us with 14 warps per SM, 11235 with 24).
+//
+// Threads per block (0: free): results do not depend on them.  The largest
+// block whose CTAs load every SM alike (40,000 runs are 157 CTAs of 256 threads,
+// two of them on five of the 152 SMs: 6.08 ms; as 128-thread CTAs 4.82 ms).
+int stepper_grid(const StepperKernel& k, int n_sets, unsigned long long n_total, const RunLengths& len, int* block,
+                 int* grid) {
     int n_sm = 0;
     int rc = device_sm_count(&n_sm);
     if (rc) return rc;
-    int per_sm = 0;
-    const size_t smem = stepper_smem(k, block, n_sets);
-    cudaError_t e = cudaFuncSetAttribute(k.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k.func, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
     if (e != cudaSuccess) return cuda_fail(e, "stepper shared memory");
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.func, block, smem);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-    if (per_sm < 1) per_sm = 1;
-    const unsigned long long full = (unsigned long long)per_sm * n_sm;
-    const unsigned long long need = (n_total + block - 1) / block;
-    *grid = (int)(need < full ? (need < 1 ? 1 : need) : full);
+    const double share = len.total / (32.0 * n_sm);
+    const bool fixed = *block != 0;
+    int best = 0;
+    // many runs: 256 threads (up to 1 % faster); fewer: 128 (3 x 45,000 equal runs 1652 us, 1774 with
+    // 256; 64 uneven sets of 16,384 runs 26.8 ms, 30.0 with 256)
+    const int first = n_total >= 32ull * kTrailingRuns ? 256 : 128;
+    for (int b = fixed ? *block : first; b >= 32; b >>= 1) {
+        const size_t smem = stepper_smem(k, b, n_sets);
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.func, b, smem);
+        if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+        const int warps = b / 32, full = per_sm * warps;
+        int r = full;
+        const double trail = share > 0.0 ? len.tail * full / share : 0.0;
+        if (trail > 0.15) r = full / 2;
+        else if (trail > 0.06) r = 3 * full / 4;
+        if (len.longest * (double)n_total > 1.5 * len.total)
+            r = std::min(r, std::max(8, (int)std::ceil(1.25 * share / len.longest)));
+        per_sm = std::max(1, r / warps);
+        const unsigned long long need = std::max(1ull, (n_total + b - 1) / b);
+        const unsigned long long room = (unsigned long long)per_sm * n_sm;
+        // warps on the fullest SM: of the only wave, else the share of the whole work that a ticket queue gives
+        const int load = need <= room ? (int)((need + n_sm - 1) / n_sm) * warps : per_sm * warps;
+        if (best == 0 || (need <= room && load < best)) {
+            best = load;
+            *block = b;
+            *grid = (int)std::min(need, room);
+        }
+        if (fixed) break;
+    }
     return FPT_OK;
 }
 
@@ -411,7 +525,7 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
     int block = 0, grid = 0;
     int rc = pick_stepper(p, P.wall, &k, &block);
     if (rc) return rc;
-    rc = stepper_grid(k, block, (int)P.sets.size(), P.n_total, &grid);
+    rc = stepper_grid(k, (int)P.sets.size(), P.n_total, P.len, &block, &grid);
     if (rc) return rc;
     StepperParams a;
     a.keys = philox_keys(seed);

@@ -43,11 +43,21 @@ int check_params(const fpt_params* p);
 // since the occupancy API is conservative for kernels that allocate TMEM.
 int resident_ctas(const void* func, int threads, size_t dyn_smem, int tmem_cols, int* per_sm);
 
+// Expected lengths of the runs of a launch, in steps: their sum, the longest set
+// and how far runs of the sets handed out last may outlast their expectation.
+struct RunLengths {
+    double total, longest, tail;
+};
+constexpr long long kTrailingRuns = 1 << 17;  // about the lanes of one GPU
+
+constexpr int kMaxDynSmem = 227 * 1024;  // opt-in limit per block
+
 // Host-side image of one batched call.
 struct Prepared {
     std::vector<SetConst> sets;
     std::vector<HistSeg> segs;
     unsigned long long n_total;
+    RunLengths len;
     bool wall;
     int max_nb;
     long long max_n;
@@ -64,11 +74,18 @@ struct WorkspaceLayout {
 
 int prepare(const fpt_params* p, const fpt_set* sets, int n_sets, bool with_hist, Prepared* P);
 int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetConst* out);
+// Hand out the tickets of the sets with the longest expected runs first: sorts
+// the table, sets each entry's first ticket (records keep their places) and
+// returns what the launch shape needs to know of the lengths.
+void order_tickets(const fpt_params* p, SetConst* table, const fpt_set* sets, int n_sets, RunLengths* len);
+// block: the caller's or the autotuned threads per block, 0 where neither is set
 int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block);
 // Launch shape chosen by fpt_autotune for this device and kind of launch, if any.
 bool tuned_shape(int precision, int model, bool wall, int* block, int* ks);
 void clear_tuned_shapes();
-int stepper_grid(const StepperKernel& k, int block, int n_sets, unsigned long long n_total, int* grid);
+// Grid of a persistent launch, and its threads per block where *block is 0.
+int stepper_grid(const StepperKernel& k, int n_sets, unsigned long long n_total, const RunLengths& len, int* block,
+                 int* grid);
 void workspace_layout(const Prepared& P, WorkspaceLayout* L);
 void workspace_image(const Prepared& P, const WorkspaceLayout& L, std::vector<unsigned char>* img);
 // Enqueues the stepper and, with bins, the histogram kernels on `stream`.

@@ -122,13 +122,15 @@ extern "C" int fpt_simulate_batch_noalloc(const fpt_params* p, const fpt_set* se
         n_total += (unsigned long long)sets[i].n_traj;
     }
     if (n_total == 0) return FPT_OK;
+    RunLengths len;
+    order_tickets(p, table, sets, n_sets, &len);
     if (!out_N || !out_logw) return fail(FPT_EINVAL, "output pointer is NULL");
 
     StepperKernel k;
     int block = 0, grid = 0;
     rc = pick_stepper(p, wall, &k, &block);
     if (rc) return rc;
-    rc = stepper_grid(k, block, n_sets, n_total, &grid);
+    rc = stepper_grid(k, n_sets, n_total, len, &block, &grid);
     if (rc) return rc;
     unsigned char* ws = nullptr;
     rc = scratch_address(&ws);

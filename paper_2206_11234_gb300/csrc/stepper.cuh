@@ -611,7 +611,7 @@ stepper_kernel(const StepperParams P) {
         s_queue + (size_t)(blockDim.x >> 5) * kQueueCap * sizeof(Entry)) + threadIdx.x;
     for (int i = threadIdx.x; i < n_sets; i += blockDim.x) {
         s_sets[i] = P.sets[i];
-        s_first[i] = P.sets[i].first;
+        s_first[i] = P.sets[i].ticket0;
     }
     if (threadIdx.x == 0) s_first[n_sets] = (long long)P.n_total;
     __syncthreads();
@@ -623,7 +623,7 @@ stepper_kernel(const StepperParams P) {
     // lane state
     bool live = false, exhausted = false;
     int set = 0;
-    unsigned long long rec = 0;  // record index (= ticket)
+    unsigned long long rec = 0;  // record index
     Real phi = (Real)0, phi_end = (Real)0, twouv = (Real)0;
     int m = 0, m_max = 0;
     PhiloxLane pl{0u, 0u, 0u};
@@ -649,7 +649,7 @@ stepper_kernel(const StepperParams P) {
                 if (t >= P.n_total) {
                     exhausted = true;
                 } else {
-                    // set of record t: the last s with first[s] <= t
+                    // set of ticket t: the last s with ticket0[s] <= t
                     int lo = 0, hi = n_sets - 1;
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
@@ -666,8 +666,9 @@ stepper_kernel(const StepperParams P) {
 #endif
                     if (!bad_set) {
                     const SetConst& S = s_sets[set];
-                    rec = t;
-                    pl = philox_lane(S.traj_offset + (t - (unsigned long long)S.first), S.set_id, P.keys);
+                    const unsigned long long i = t - (unsigned long long)s_first[lo];  // run of the set
+                    rec = (unsigned long long)S.first + i;
+                    pl = philox_lane(S.traj_offset + i, S.set_id, P.keys);
                     model.load(S);
                     phi = set_phi_in<Real, MODEL>(S);
                     phi_end = set_phi_end<Real, MODEL>(S);
@@ -677,8 +678,8 @@ stepper_kernel(const StepperParams P) {
                     W.reset();
                     if (S.phi_in <= S.phi_end) {
                         // starts at or below the end of inflation: N = 0, w = 1
-                        P.out_N[t] = 0.0;
-                        P.out_logw[t] = 0.0;
+                        P.out_N[rec] = 0.0;
+                        P.out_logw[rec] = 0.0;
                     } else {
                         live = true;
                     }

@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
     }
     for (int i = tid; i < n_sets; i += blockDim.x) {
         s_sets[i] = P.sets[i];
-        s_first[i] = P.sets[i].first;
+        s_first[i] = P.sets[i].ticket0;
     }
     if (tid == 0) s_first[n_sets] = (long long)P.n_total;
     mlp_tile_load(F, W);  // ends with __syncthreads
@@ -199,8 +199,9 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
                     }
                     set = lo;
                     const SetConst& S = s_sets[set];
-                    rec = t;
-                    pl = philox_lane(S.traj_offset + (t - (unsigned long long)S.first), S.set_id, P.keys);
+                    const unsigned long long i = t - (unsigned long long)s_first[lo];  // run of the set
+                    rec = (unsigned long long)S.first + i;
+                    pl = philox_lane(S.traj_offset + i, S.set_id, P.keys);
                     model.load(S);
                     phi = S.f_phi_in;
                     phi_end = S.f_phi_end;
@@ -209,8 +210,8 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
                     m_max = S.m_max;
                     lw = 0.0;
                     if (S.phi_in <= S.phi_end) {
-                        P.out_N[t] = 0.0;
-                        P.out_logw[t] = 0.0;
+                        P.out_N[rec] = 0.0;
+                        P.out_logw[rec] = 0.0;
                     } else {
                         live = true;
                     }

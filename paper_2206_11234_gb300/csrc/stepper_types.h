@@ -20,12 +20,13 @@ __host__ __device__ constexpr bool is_pow_model(int model) { return model >= kMo
 // Per parameter set, prepared on the host (binary64 originals and the
 // binary32 step constants), copied to shared memory by every block.
 struct SetConst {
-    double phi_in, phi_end, phi_uv, twouv;  // twouv = 2 phi_uv (reflection phi -> 2 phi_uv - phi)
+    double phi_in, phi_end, twouv;          // twouv = 2 phi_uv (reflection phi -> 2 phi_uv - phi)
     double dN, sq, b;                       // sq = sqrt(dN)
     double cm;                              // quadratic: c0 m, c0 = 1/(2 pi sqrt 6); constant model: s0
     double a0;                              // constant model drift
     double lw_bsq, lw_half_b2dN;            // ln w = -lw_bsq * W - lw_half_b2dN * M
     long long first;                        // index of this set's first record
+    long long ticket0;                      // this set's first ticket (tables are in ticket order)
     unsigned long long traj_offset;         // Philox id of this set's first run
     int m_max;                              // censoring cap in steps
     uint32_t set_id;                        // Philox counter word 3

@@ -1,0 +1,86 @@
+"""Records do not depend on how a launch is laid out: the order in which the
+sets' tickets are handed out, the threads per block and the resident warps the
+library picks for a given number of runs, or the scheduling block the
+binary32 stepper works in.
+
+Sets of very different lengths (so that their tickets are reordered), with an
+empty set and one that starts at its end, must leave the records of one call
+per set, bit for bit; every block size gives the same records at run counts
+around warp, block and wave edges; and first-passage times do not depend on
+k_steps, which only sets where ln w is rounded.
+"""
+import math
+
+import numpy as np
+import pytest
+
+from paper_2206_11234_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nat(cuda_device):
+    from paper_2206_11234_gb300 import native
+    return native
+
+
+def batch(nat, specs, precision, **kw):
+    import torch
+    n = sum(s.n_traj for s in specs)
+    N = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+    lw = torch.full_like(N, -1.0)
+    nat.fpt_simulate_batch(nat.make_params(precision=precision, m=specs[0].m, n_max=specs[0].n_max, **kw),
+                           nat.make_sets(specs), 3, N, lw)
+    return N, lw
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32_kahan", "f32_f64acc"])
+def test_sets_of_rising_length_equal_one_call_per_set(nat, precision):
+    import torch
+    spec = dict(dN=2e-3, n_max=8.0)
+    specs = [W.SetSpec(phi_in=1.6, m=0.1, b=0.0, n_traj=333, set_id=0, **spec),
+             W.SetSpec(phi_in=3.0, m=1.0, b=0.0, n_traj=0, set_id=1, **spec),
+             W.SetSpec(phi_in=2.5, m=1.0, b=1.0, n_traj=1025, set_id=2, phi_uv=2.6, **spec),
+             W.SetSpec(phi_in=1.2, m=1.0, b=0.0, n_traj=65, set_id=3, **spec),  # starts past the end: N = 0
+             W.SetSpec(phi_in=4.0, m=1.0, b=30.0, n_traj=129, set_id=4, **spec),  # escapes: censored
+             W.SetSpec(phi_in=4.0, m=0.01, b=0.0, n_traj=31, set_id=5, **spec)]
+    N, lw = batch(nat, specs, precision)
+    off = 0
+    for s in specs:
+        if s.n_traj:
+            N1, l1 = batch(nat, [s], precision)
+            # the wall of another set makes the kernel mirror at infinity too, which changes nothing
+            assert torch.equal(N[off:off + s.n_traj], N1), s.set_id
+            assert torch.equal(lw[off:off + s.n_traj], l1), s.set_id
+        off += s.n_traj
+    assert torch.all(N[-31 - 129 - 65:-31 - 129] == 0.0)
+    assert torch.all(torch.isinf(N[-31 - 129:-31]))
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32_kahan"])
+@pytest.mark.parametrize("n", [1, 31, 33, 4865, 20001])
+def test_any_block_size_gives_the_same_records(nat, precision, n):
+    import torch
+    s = W.SetSpec(phi_in=1.8, m=1.0, b=0.5, dN=2e-3, n_max=3.0, n_traj=n)
+    N, lw = batch(nat, [s], precision)
+    for block in (32, 96, 512):
+        N1, l1 = batch(nat, [s], precision, block_dim=block)
+        assert torch.equal(N, N1) and torch.equal(lw, l1), block
+
+
+@pytest.mark.parametrize("precision", ["f32_kahan", "f32_f64acc"])
+@pytest.mark.parametrize("n_max", [0.002, 0.03, 0.034, 0.128, 0.13, 3.0])
+def test_block_lengths_agree(nat, precision, n_max):
+    """Caps below, at and past 16- and 64-step edges; ln w agrees to the
+    rounding of its binary32 block sums (at most 64 terms of a few units each:
+    64 x 4 x 2^-24 x b sqrt(dN) per block, and at most n_max / dN / 16 blocks)."""
+    dN, b = 2e-3, 0.5
+    s = W.SetSpec(phi_in=1.45, m=1.0, b=b, dN=dN, n_max=n_max, n_traj=5000)
+    N, lw = batch(nat, [s], precision)
+    steps = math.ceil(n_max / dN)
+    tol = 64 * 4 * 2.0 ** -24 * b * math.sqrt(dN) * math.ceil(steps / 16)
+    for ks in (16, 32, 64):
+        N1, l1 = batch(nat, [s], precision, k_steps=ks)
+        assert np.array_equal(N.cpu().numpy(), N1.cpu().numpy()), ks
+        assert float((lw - l1).abs().max()) <= tol, ks
