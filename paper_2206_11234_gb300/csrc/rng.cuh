@@ -179,6 +179,13 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 __device__ __forceinline__ uint32_t angle_word_first(uint32_t ang) { return ang & 0xffff0000u; }
 __device__ __forceinline__ uint32_t angle_word_second(uint32_t ang) { return __byte_perm(ang, 0u, 0x1044); }
 
+// lg2.approx of a normal binary32 number
+__device__ __forceinline__ float lg2_approx(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 struct NormalPair {
     float rho;  // sqrt(-log2 u0)
     float c;    // cos(2 pi u1 - pi)
@@ -187,7 +194,7 @@ struct NormalPair {
 
 __device__ __forceinline__ NormalPair normal_pair_f32(uint32_t rad, uint32_t angle_word) {
     NormalPair p;
-    p.rho = sqrt_approx(-__log2f(uniform_f32(rad)));
+    p.rho = sqrt_approx(-lg2_approx(uniform_f32(rad)));  // u0 >= 2^-24: never subnormal
     const float f = __int_as_float((angle_word >> 9) + 0x3f800000u);
     const float angle = __fmaf_rn(6.283185307179586f, f, -kAngleOffset);
     __sincosf(angle, &p.s, &p.c);

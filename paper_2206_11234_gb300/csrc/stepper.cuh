@@ -36,11 +36,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float lg2_approx(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -238,9 +233,13 @@ __device__ __forceinline__ void quad_block_f32(const Step& model, const uint32_t
 // of group g, so that a warp's instruction stream interleaves the integer
 // multiplies with the XU work instead of alternating between the two phases.
 // The words, and so the results, are those of computing each group in turn.
-template <int KS, typename Block>
+// group_end(g) follows the last block of group g.
+struct NoGroupEnd {
+    __device__ __forceinline__ void operator()(int) const {}
+};
+template <int KS, typename Block, typename GroupEnd = NoGroupEnd>
 __device__ __forceinline__ void pipelined_groups(const PhiloxLane& pl, uint32_t G0, const PhiloxKeys& keys,
-                                                 Block&& block) {
+                                                 Block&& block, GroupEnd&& group_end = GroupEnd{}) {
     static_assert(KS % 16 == 0, "whole 16-step groups");
     uint32_t V[12];
     philox_group(pl, G0, keys, V);
@@ -253,6 +252,7 @@ __device__ __forceinline__ void pipelined_groups(const PhiloxLane& pl, uint32_t 
                 philox_block(pl, 3u * (G0 + (uint32_t)g + 1u) + (uint32_t)j, keys, Vn + 4 * j);
             block(V, j);
         }
+        group_end(g);
         if (g + 1 < KS / 16) {
 #pragma unroll
             for (int i = 0; i < 12; ++i) V[i] = Vn[i];
@@ -362,6 +362,10 @@ struct WSum<FPT_PREC_F32_KAHAN> {
         c = __fsub_rn(__fsub_rn(t, s), y);
         s = t;
     }
+    __device__ __forceinline__ void take(const WSum& o, bool yes) {
+        s = yes ? o.s : s;
+        c = yes ? o.c : c;
+    }
     __device__ __forceinline__ double total(float tail) const {
         return ((double)s - (double)c) + (double)tail;
     }
@@ -372,6 +376,7 @@ struct WSum<FPT_PREC_F32_F64ACC> {
     double s;
     __device__ __forceinline__ void reset() { s = 0.0; }
     __device__ __forceinline__ void add(float x) { s += (double)x; }
+    __device__ __forceinline__ void take(const WSum& o, bool yes) { s = yes ? o.s : s; }
     __device__ __forceinline__ double total(float tail) const { return s + (double)tail; }
 };
 
@@ -419,14 +424,16 @@ __device__ __forceinline__ Real set_twouv(const SetConst& S) {
     else return S.f_twouv;
 }
 
-// A run that finished inside its last block, waiting for the replay.
+// A run that finished inside its last block, waiting for the replay.  The state
+// is that of the last fold before its end (binary32) or of the start of the
+// block in which it finished (binary64).
 template <typename Real, int PREC>
 struct Pending {
     unsigned long long rec;  // record index
-    int m0;                  // step count at the block start
+    int m0;                  // step count there
     int set;                 // parameter set
-    Real phi0;               // phi at the block start
-    WSum<PREC> W;            // running sum of the normals before the block
+    Real phi0;               // phi there
+    WSum<PREC> W;            // running sum of the normals up to there
 };
 
 constexpr int kQueueCap = 64;  // per warp: up to 31 waiting + 32 new
@@ -489,7 +496,7 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
     int M = 0;
     bool crossed = false;
     if constexpr (sizeof(Real) == 4) {
-        // binary32: whole 16-step groups, as the stepping loop draws them
+        // binary32: the 16-step groups from there, as the stepping loop draws them
         for (int gg = 0; gg < KS / 16; ++gg) {
             uint32_t V[12];
             philox_group(pl, ((uint32_t)e.m0 >> 4) + (uint32_t)gg, P.keys, V);
@@ -593,7 +600,11 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
 #ifndef FPT_STEPPER_MAXNREG
 #define FPT_STEPPER_MAXNREG 64
 #endif
-template <typename Real, int PREC, int MODEL, bool WALL, int KS>
+//
+// KS: steps of a scheduling block.  FOLD (binary32): the sum of the normals is
+// folded into the running sum W every FOLD steps; that sets the rounding of ln w,
+// so it is what a caller's k_steps chooses, while the block length is free.
+template <typename Real, int PREC, int MODEL, bool WALL, int KS, int FOLD>
 __global__ void __maxnreg__(FPT_STEPPER_MAXNREG)
 stepper_kernel(const StepperParams P) {
     static_assert(KS % (sizeof(Real) == 4 ? 16 : 4) == 0,
@@ -690,22 +701,40 @@ stepper_kernel(const StepperParams P) {
         if (!__any_sync(FULL, live)) break;
 
         // ---- one scheduling block of KS steps, no per-step branches ----
-        const Real phi0 = phi;
-        const int m0 = m;
+        Real phi0 = phi;
+        int m0 = m;
         Real mn = phi;
         Real sblk = (Real)0;
+        bool event;
         if constexpr (sizeof(Real) == 4) {
-            const uint32_t G0 = (uint32_t)m0 >> 4;
+            static_assert(KS % FOLD == 0 && FOLD % 16 == 0, "whole groups per fold, whole folds per block");
+            const uint32_t G0 = (uint32_t)m >> 4;
+            bool on = true;  // the run has not finished yet in this block
+            // every FOLD steps a run that is still on folds its sum and commits (phi, m):
+            // what a finished run leaves is the state at the last fold before its end
+            auto group_end = [&](int g) {
+                const int mg = m + 16 * (g + 1);
+                if ((16 * (g + 1)) % FOLD != 0) return;
+                on = !(mn <= phi_end) && mg < m_max;
+                WSum<PREC> Wn = W;
+                Wn.add(sblk);
+                W.take(Wn, on);
+                sblk = 0.f;
+                phi0 = on ? phi : phi0;
+                m0 = on ? mg : m0;
+            };
             if constexpr (is_pow_model(MODEL))
                 pipelined_groups<KS>(pl, G0, P.keys, [&](const uint32_t* V, int j) {
                     pow_block_f32<MODEL, WALL>(model, V, j, twouv, phi, mn, sblk);
-                });
+                }, group_end);
             else
                 pipelined_groups<KS>(pl, G0, P.keys, [&](const uint32_t* V, int j) {
                     quad_block_f32<WALL>(model, V, j, twouv, phi, mn, sblk);
-                });
+                }, group_end);
+            m += KS;
+            event = live && !on;
         } else {
-            const uint32_t k0 = (uint32_t)m0 >> 2;
+            const uint32_t k0 = (uint32_t)m >> 2;
 #pragma unroll
             for (int g = 0; g < KS / 4; ++g) {
                 Real xi[4];
@@ -722,12 +751,13 @@ stepper_kernel(const StepperParams P) {
                     mn = real_min<Real>(mn, phi);
                 }
             }
+            m += KS;
+            event = live && (mn <= phi_end || m >= m_max);
+            if (live && !event) W.add(sblk);
         }
-        m = m0 + KS;
-        const bool event = live && (mn <= phi_end || m >= m_max);
         const unsigned ev = __ballot_sync(FULL, event);
         if (ev) {
-            // finished inside this block: queue the block-start state, free the lane
+            // finished inside this block: queue the committed state, free the lane
             if (event) {
                 const int at = q_count + __popc(ev & lt_mask);
 #if FPT_DEBUG
@@ -763,7 +793,7 @@ stepper_kernel(const StepperParams P) {
                 park(v, 9 * stride, pl.r1_x1);
                 park(v, 10 * stride, pl.r1_set);
                 __syncwarp();
-                replay_batch<Real, PREC, MODEL, WALL, KS>(q, 32, P, s_sets, lane, my_steps);
+                replay_batch<Real, PREC, MODEL, WALL, sizeof(Real) == 4 ? FOLD : KS>(q, 32, P, s_sets, lane, my_steps);
                 __syncwarp();
                 const int rest = q_count - 32;
                 Entry tmp;
@@ -792,11 +822,10 @@ stepper_kernel(const StepperParams P) {
                 m_max = S.m_max;
             }
         }
-        if (live) W.add(sblk);
     }
     if (q_count > 0) {
         __syncwarp();
-        replay_batch<Real, PREC, MODEL, WALL, KS>(q, q_count, P, s_sets, lane, my_steps);
+        replay_batch<Real, PREC, MODEL, WALL, sizeof(Real) == 4 ? FOLD : KS>(q, q_count, P, s_sets, lane, my_steps);
     }
 
     // ---- total steps: warp reduce, one atomic per warp ----

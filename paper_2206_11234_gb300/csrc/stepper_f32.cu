@@ -5,17 +5,19 @@
 namespace fpt {
 namespace {
 
-template <int PREC, int MODEL, bool WALL, int KS>
+constexpr int kBlock32 = 64;  // steps of a scheduling block, whatever k_steps folds
+
+template <int PREC, int MODEL, bool WALL, int FOLD>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) + (size_t)(block / 32) * warp_smem_bytes<float, PREC>();
-    stepper_kernel<float, PREC, MODEL, WALL, KS><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
-template <int PREC, int MODEL, bool WALL, int KS>
+template <int PREC, int MODEL, bool WALL, int FOLD>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, KS>,
-                         warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, KS>};
+    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD>,
+                         warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, FOLD>};
 }
 
 template <int PREC, int MODEL, bool WALL>

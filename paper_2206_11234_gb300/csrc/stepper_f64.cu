@@ -11,13 +11,13 @@ namespace {
 template <int MODEL, bool WALL, int KS>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) + (size_t)(block / 32) * warp_smem_bytes<double, FPT_PREC_F64>();
-    stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS, KS><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
 template <int MODEL, bool WALL, int KS>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS>,
+    return StepperKernel{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS, KS>,
                          warp_smem_bytes<double, FPT_PREC_F64>(), &launch<MODEL, WALL, KS>};
 }
 

@@ -12,13 +12,13 @@ constexpr int kPowKS = 32;
 template <int PREC, int MODEL, bool WALL>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) + (size_t)(block / 32) * warp_smem_bytes<float, PREC>();
-    stepper_kernel<float, PREC, MODEL, WALL, kPowKS><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
 template <int PREC, int MODEL, bool WALL>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, kPowKS>,
+    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS>,
                          warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL>};
 }
 
