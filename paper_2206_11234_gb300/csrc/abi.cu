@@ -411,7 +411,13 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
         *k = stepper_f64(p->model, wall, s);
     } else {
         if (s == 0) s = 16;
-        *k = stepper_f32(p->precision, p->model, wall, s);
+        int model = p->model;
+        if (model == FPT_MODEL_POLYNOMIAL) {
+            bool quartic = true;
+            for (int i = kPolyLow + 1; i < FPT_POLY_TERMS; ++i) quartic = quartic && p->poly[i] == 0.0;
+            if (quartic) model = kModelPolyLow;
+        }
+        *k = stepper_f32(p->precision, model, wall, s);
     }
     if (!k->func) return fail(FPT_EINVAL, "k_steps %d not available for precision %d", s, p->precision);
     *block = b;

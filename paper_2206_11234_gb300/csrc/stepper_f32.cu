@@ -40,6 +40,7 @@ StepperKernel by_model(int model, bool wall, int ks) {
     if (model == FPT_MODEL_QUADRATIC) return by_wall<PREC, FPT_MODEL_QUADRATIC>(wall, ks);
     if (model == FPT_MODEL_CONSTANT) return by_wall<PREC, FPT_MODEL_CONSTANT>(wall, ks);
     if (model == FPT_MODEL_POLYNOMIAL) return by_wall<PREC, FPT_MODEL_POLYNOMIAL>(wall, ks);
+    if (model == kModelPolyLow) return by_wall<PREC, kModelPolyLow>(wall, ks);
     return StepperKernel{nullptr, 0, nullptr};
 }
 

@@ -15,6 +15,9 @@ constexpr int kStepperMaxThreads = 512;
 // multiplies), kModelPowReal for any real p (phi^(p-1) = 2^((p-1) log2 phi)).
 constexpr int kModelPow = 16;
 constexpr int kModelPowReal = kModelPow + 15;
+// Model tag of a polynomial potential of degree at most kPolyLow (binary32 kernels).
+constexpr int kPolyLow = 4;
+constexpr int kModelPolyLow = 8;
 __host__ __device__ constexpr bool is_pow_model(int model) { return model >= kModelPow; }
 
 // Per parameter set, prepared on the host (binary64 originals and the

@@ -84,3 +84,21 @@ def test_block_lengths_agree(nat, precision, n_max):
         N1, l1 = batch(nat, [s], precision, k_steps=ks)
         assert np.array_equal(N.cpu().numpy(), N1.cpu().numpy()), ks
         assert float((lw - l1).abs().max()) <= tol, ks
+
+
+@pytest.mark.parametrize("precision", ["f32_kahan", "f32_f64acc"])
+@pytest.mark.parametrize("c", [[0, 0, 0, 0, 0.0125], [0.02, 0, 0.1, 0.01], [0, 0, 0.15, 0, 0.005]])
+@pytest.mark.parametrize("phi_uv", [math.inf, 4.6])
+def test_low_degree_polynomial_is_the_general_one(nat, precision, c, phi_uv):
+    """A potential of degree <= 4 starts Horner's rule at its own degree; with a
+    coefficient of phi^7 that is zero in binary32 only, the general kernel runs
+    the same potential: the same records, bit for bit."""
+    import torch
+    out = []
+    for poly in (c, c + [0.0] * (7 - len(c)) + [1e-300]):
+        N = torch.empty(4097, dtype=torch.float64, device="cuda")
+        lw = torch.empty_like(N)
+        p = nat.make_params(model=nat.MODEL_POLYNOMIAL, precision=precision, poly=poly, n_max=6.0)
+        nat.fpt_simulate(p, N.numel(), 4.0, 2.5, phi_uv, 1e-3, 0.6, 9, N, lw)
+        out.append((N, lw))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
