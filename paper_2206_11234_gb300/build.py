@@ -15,6 +15,7 @@ variable FPT_DEBUG_LIB is 1.
 import concurrent.futures as cf
 import os
 import shutil
+import struct
 import subprocess
 import sys
 
@@ -44,6 +45,67 @@ UNITS = {
     "pipes.cu": [],
     "hist_merge.cu": [],
 }
+
+
+def f64_tables() -> str:
+    """The binary64 Box–Muller tables of csrc/rng64.cuh, rounded correctly from
+    200-bit integer arithmetic: cosines and sines of the 2^16 angles 2 pi u1 (the
+    binary64 product), the logarithm's 2^-20-grained reciprocals with 2 ln(2 inv),
+    and the multiples of 2 ln 2."""
+    bits = 200
+    one = 1 << bits
+
+    def series(n, odd_sign):  # atan(1/n) (odd_sign -1) or atanh(1/n) (odd_sign 1)
+        t = one // n
+        s, k, sign = t, 1, 1
+        while t:
+            t //= n * n
+            k += 2
+            sign *= odd_sign
+            s += sign * (t // k)
+        return s
+
+    pi = 4 * (4 * series(5, -1) - series(239, -1))  # Machin
+    ln2 = 2 * series(3, 1)
+
+    def cos_sin(x):
+        out = [0, 0]
+        t, k = one, 0
+        while t:
+            out[k % 2] += t if k % 4 < 2 else -t
+            k += 1
+            t = (t * x >> bits) // k
+        return out
+
+    def ln_ratio(a, b):  # ln(a / b) = 2 atanh((a - b) / (a + b)), 1 <= a / b <= 2
+        z = (a - b) * one // (a + b)
+        z2 = z * z >> bits
+        s, t, k = 0, z, 1
+        while t:
+            s += t // k
+            t = t * z2 >> bits
+            k += 2
+        return 2 * s
+
+    c, s = cos_sin(pi >> 16)
+    dc, ds = cos_sin(pi >> 15)
+    trig = []
+    for h in range(1 << 16):
+        num, den = (6.283185307179586 * ((h + 0.5) / 65536)).as_integer_ratio()
+        e = num * one // den - (pi * (2 * h + 1) >> 16)  # the rounded angle less the angle
+        trig.append(((c - (s * e >> bits)) / one, (s + (c * e >> bits)) / one))  # int / int rounds correctly
+        c, s = (c * dc - s * ds) >> bits, (s * dc + c * ds) >> bits
+    log = []
+    for i in range(1 << 10):
+        inv = ((1 << 21) * (1 << 11) // (2 * (1 << 10) + 2 * i + 1) + 1) >> 1  # 2^20 / (1 + (i + 1/2)/1024), rounded
+        if i == (1 << 10) - 1:
+            inv = 1 << 19  # exactly 1/2 next to u0 = 1
+        log.append((-2.0 * inv / (1 << 20), 2 * ln_ratio(inv, 1 << 19) / one))
+    word = lambda x: "0x%xull" % struct.unpack("<Q", struct.pack("<d", x))  # noqa: E731
+    pairs = lambda rows: ",".join("{%s,%s}" % (word(a), word(b)) for a, b in rows)  # noqa: E731
+    return ("__device__ const ulonglong2 kTrig64[65536] = {%s};\n__device__ const ulonglong2 kLog64[1024] = {%s};\n"
+            "__device__ const unsigned long long kLn2N64[33] = {%s};\n"
+            % (pairs(trig), pairs(log), ",".join(word(2 * n * ln2 / one) for n in range(33))))
 
 
 def nvcc() -> str:
@@ -81,12 +143,14 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
         return lib
     build_dir = BUILD + ("_debug" if debug else "")
     os.makedirs(build_dir, exist_ok=True)
+    with open(os.path.join(build_dir, "f64_tables.inc"), "w") as f:
+        f.write(f64_tables())
     cc = nvcc()
     extra = ["-DFPT_DEBUG=1"] if debug else []
 
     def compile_unit(name):
         obj = os.path.join(build_dir, name.replace(".cu", ".o"))
-        cmd = [cc, *ARCH, *COMMON, *extra, *UNITS[name], "-c", os.path.join(CSRC, name), "-o", obj]
+        cmd = [cc, *ARCH, *COMMON, "-I" + build_dir, *extra, *UNITS[name], "-c", os.path.join(CSRC, name), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         r = subprocess.run(cmd, capture_output=True, text=True)

@@ -252,6 +252,13 @@ int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetCo
         c.f_c2 = (float)(neg_sqrt2ln2 * c.sq);               // noise part of dphi / S per unit rho cos
         c.f_c3 = (float)s.dN;
     } else if (p->model == FPT_MODEL_QUADRATIC) {
+        if (p->precision == FPT_PREC_F64) {
+            c.d_psi_in = psi_per_phi * s.phi_in;
+            c.d_psi_end = psi_per_phi * s.phi_end;
+            c.d_psi_twouv = psi_per_phi * c.twouv;
+            c.d_c1 = s.b * c.cm * s.dN;
+            c.d_c2 = c.cm * c.sq;
+        }
         c.f_c1 = (float)(s.b * c.cm * s.dN);                 // bias part of dphi/phi
         c.f_c2 = (float)(neg_sqrt2ln2 * c.cm * c.sq);        // noise part of dphi/phi per unit rho cos
         c.f_c3 = (float)(-2.0 * s.dN);                       // drift part of dphi, times phi

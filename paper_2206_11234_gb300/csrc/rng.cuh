@@ -127,27 +127,6 @@ __device__ __forceinline__ void philox4x32_10(const uint32_t c[4], uint32_t key0
     w[3] = x3;
 }
 
-// ---- Box–Muller, binary64: u0 = (w + 1/2) 2^-32 from a radius word, u1 =
-// (h + 1/2) 2^-16 from a 16-bit angle field (both exact), r = sqrt(-2 ln u0),
-// (r cos 2 pi u1, r sin 2 pi u1) with CUDA's log, sqrt and sincos. ----
-__device__ __forceinline__ void box_muller_f64(uint32_t rad, uint32_t ang16, double& z0, double& z1) {
-    const double u0 = ((double)rad + 0.5) * 0x1p-32;
-    const double u1 = ((double)ang16 + 0.5) * 0x1p-16;
-    const double r = sqrt(-2.0 * log(u0));
-    const double angle = 6.283185307179586 * u1;
-    double s, c;
-    sincos(angle, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
-}
-
-__device__ __forceinline__ void normals4_f64(const PhiloxLane& l, uint32_t k, const PhiloxKeys& K,
-                                             double xi[4]) {
-    const BlockWords w = block_words(l, k, K);
-    box_muller_f64(w.rad0, w.ang >> 16, xi[0], xi[1]);
-    box_muller_f64(w.rad1, w.ang & 0xffffu, xi[2], xi[3]);
-}
-
 // ---- Box–Muller, binary32 (hardware approximations) ----
 // u0 = ((w >> 9) + 1/2) 2^-23 is exact in binary32: put the top 23 bits of the
 // radius word into the mantissa of 1.0 (a shift-add, the bits do not overlap)

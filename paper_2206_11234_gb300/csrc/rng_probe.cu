@@ -5,7 +5,7 @@
 
 #include "abi_internal.h"
 #include "fpt.h"
-#include "rng.cuh"
+#include "rng64.cuh"
 
 namespace fpt {
 namespace {

@@ -27,6 +27,7 @@
 #include <cstdint>
 
 #include "rng.cuh"
+#include "rng64.cuh"
 #include "stepper_types.h"
 
 namespace fpt {
@@ -84,6 +85,7 @@ struct ModelStep<float, FPT_MODEL_QUADRATIC> {
 // multiply.  The increment is still formed on its own (one rounding) and then
 // added.  Crossing and wall tests compare psi with the scaled phi_end and
 // 2 phi_uv of the set table; the crossing fraction is scale-free.
+struct QuadPsiStep64;  // the same in binary64, below
 struct QuadPsiStep {
     float tc, kq;  // as in ModelStep<float, FPT_MODEL_QUADRATIC>
     __device__ __forceinline__ void load(const SetConst& s) {
@@ -189,6 +191,8 @@ template <typename Real, int MODEL>
 struct StepOf { using type = ModelStep<Real, MODEL>; };
 template <>
 struct StepOf<float, FPT_MODEL_QUADRATIC> { using type = QuadPsiStep; };
+template <>
+struct StepOf<double, FPT_MODEL_QUADRATIC> { using type = QuadPsiStep64; };
 
 // Sixteen binary32 EM steps of a power model from one Philox group: as
 // Block j (four steps, two Box–Muller pairs) of a 16-step group for the
@@ -272,23 +276,20 @@ __device__ __forceinline__ void pipelined_groups(const PhiloxLane& pl, uint32_t 
 // The binary32 sums are kept in units of -1/sqrt(2 ln 2) of the sum of the normals.
 constexpr double kXiPerRho = -1.1774100225154747;  // -sqrt(2 ln 2)
 
-// Binary64 (reference) steps: the update exactly as written in Eq. (11).  This
-// translation unit is compiled without FMA contraction, so each operation is
-// rounded as written.
-template <>
-struct ModelStep<double, FPT_MODEL_QUADRATIC> {
-    double cm, b, dN, sq;
+// Binary64 (reference) steps.  This translation unit is compiled without FMA
+// contraction: the constant, polynomial and power models round each operation
+// as written.  The quadratic step is written out with its fused operations: in
+// psi, as the binary32 one, psi' = psi + (psi t - 1/psi) with t = c2 xi + c1, five
+// binary64 instructions and one for t (as written in Eq. (11), with the library's
+// division, about 17) and no rounding more.
+struct QuadPsiStep64 {
+    double tc, kq;  // b c m dN, c m sqrt(dN)
     __device__ __forceinline__ void load(const SetConst& s) {
-        cm = s.cm;
-        b = s.b;
-        dN = s.dN;
-        sq = s.sq;
+        tc = s.d_c1;
+        kq = s.d_c2;
     }
-    __device__ __forceinline__ double step(double phi, double xi) const {
-        const double D = -2.0 / phi;
-        const double S = cm * phi;
-        const double B = b * S;
-        return phi + (D + B) * dN + S * xi * sq;
+    __device__ __forceinline__ double step(double psi, double t) const {
+        return __dadd_rn(psi, __fma_rn(psi, t, -reciprocal(psi)));
     }
 };
 
@@ -394,48 +395,92 @@ struct WSum<FPT_PREC_F64> {
     double s;
     __device__ __forceinline__ void reset() { s = 0.0; }
     __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void take(const WSum& o, bool yes) { s = yes ? o.s : s; }
     __device__ __forceinline__ double total(double tail) const { return s + tail; }
 };
 
-template <typename Real>
-__device__ __forceinline__ void normals4(const PhiloxLane& l, uint32_t k, const PhiloxKeys& K, Real xi[4]);
+__device__ __forceinline__ float real_min(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ double real_min(double a, double b) { return fmin(a, b); }
+
+// Whether any state of a block was at or below phi_end (binary64).  A binary64
+// minimum or comparison occupies the binary64 pipe like an addition; the
+// quadratic model, whose psi_end is positive, compares bit patterns as integers
+// instead (negative states lie below, NaN counts as not reached, as in fmin).
+template <int MODEL>
+struct Reached64 {
+    double lowest, end;
+    __device__ __forceinline__ void reset(double x, double e) {
+        lowest = x;
+        end = e;
+    }
+    __device__ __forceinline__ void see(double x) { lowest = fmin(lowest, x); }
+    __device__ __forceinline__ bool any() const { return lowest <= end; }
+};
 template <>
-__device__ __forceinline__ void normals4<double>(const PhiloxLane& l, uint32_t k, const PhiloxKeys& K,
-                                                 double xi[4]) {
-    normals4_f64(l, k, K, xi);
+struct Reached64<FPT_MODEL_QUADRATIC> {
+    bool hit;
+    int hi;
+    unsigned lo;
+    __device__ __forceinline__ void reset(double, double e) {
+        hit = false;
+        hi = __double2hiint(e);
+        lo = (unsigned)__double2loint(e);
+    }
+    __device__ __forceinline__ void see(double x) {
+        const int h = __double2hiint(x);
+        const bool below = h < hi || (h == hi && (unsigned)__double2loint(x) <= lo);
+        hit = hit || (below && ((unsigned)h << 1) <= 0xffe00000u);
+    }
+    __device__ __forceinline__ bool any() const { return hit; }
+};
+
+// One Box–Muller pair of binary64 steps: after(phi) follows each step.
+template <int MODEL, bool WALL, typename Step, typename After>
+__device__ __forceinline__ void pair_steps_f64(const Step& model, const PairF64& np, double twouv, double& phi,
+                                               double& acc, After&& after) {
+    double q = np.r;
+    if constexpr (MODEL == FPT_MODEL_QUADRATIC) q = __dmul_rn(q, model.kq);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const double trig = h == 0 ? np.c : np.s;
+        if constexpr (MODEL == FPT_MODEL_QUADRATIC) {
+            phi = model.step(phi, __fma_rn(q, trig, model.tc));
+            acc = __fma_rn(np.r, trig, acc);
+        } else if constexpr (is_pow_model(MODEL)) {
+            phi = model.advance(phi, __dmul_rn(q, trig), acc);
+        } else {
+            const double xi = __dmul_rn(q, trig);
+            phi = model.step(phi, xi);
+            acc = __dadd_rn(acc, xi);
+        }
+        if constexpr (WALL) phi = real_min(phi, twouv - phi);  // mirror at phi_uv
+        if (after(phi, h)) return;
+    }
 }
 
-template <typename Real>
-__device__ __forceinline__ Real real_min(Real a, Real b);
-template <>
-__device__ __forceinline__ float real_min<float>(float a, float b) { return fminf(a, b); }
-template <>
-__device__ __forceinline__ double real_min<double>(double a, double b) { return fmin(a, b); }
-
-// phi_in, phi_end and 2 phi_uv in the stepper's state variable: binary64 phi,
-// binary32 phi, or binary32 psi = phi / sqrt(2 dN) for the quadratic constant-bias step
+// phi_in, phi_end and 2 phi_uv in the stepper's state variable: phi, or
+// psi = phi / sqrt(2 dN) for the quadratic constant-bias step
 template <typename Real, int MODEL>
 __device__ __forceinline__ Real set_phi_in(const SetConst& S) {
-    if constexpr (sizeof(Real) == 8) return (Real)S.phi_in;
+    if constexpr (sizeof(Real) == 8) return MODEL == FPT_MODEL_QUADRATIC ? S.d_psi_in : S.phi_in;
     else if constexpr (MODEL == FPT_MODEL_QUADRATIC) return S.f_psi_in;
     else return S.f_phi_in;
 }
 template <typename Real, int MODEL>
 __device__ __forceinline__ Real set_phi_end(const SetConst& S) {
-    if constexpr (sizeof(Real) == 8) return (Real)S.phi_end;
+    if constexpr (sizeof(Real) == 8) return MODEL == FPT_MODEL_QUADRATIC ? S.d_psi_end : S.phi_end;
     else if constexpr (MODEL == FPT_MODEL_QUADRATIC) return S.f_psi_end;
     else return S.f_phi_end;
 }
 template <typename Real, int MODEL>
 __device__ __forceinline__ Real set_twouv(const SetConst& S) {
-    if constexpr (sizeof(Real) == 8) return (Real)S.twouv;
+    if constexpr (sizeof(Real) == 8) return MODEL == FPT_MODEL_QUADRATIC ? S.d_psi_twouv : S.twouv;
     else if constexpr (MODEL == FPT_MODEL_QUADRATIC) return S.f_psi_twouv;
     else return S.f_twouv;
 }
 
 // A run that finished inside its last block, waiting for the replay.  The state
-// is that of the last fold before its end (binary32) or of the start of the
-// block in which it finished (binary64).
+// is that of the last fold before its end.
 template <typename Real, int PREC>
 struct Pending {
     unsigned long long rec;  // record index
@@ -541,28 +586,21 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
             if (__all_sync(mask, M != 0)) break;
         }
     } else {
-        const uint32_t k0 = (uint32_t)e.m0 >> 2;
         for (int g = 0; g < KS / 4; ++g) {
-            Real xi[4];
-            normals4<Real>(pl, k0 + (uint32_t)g, P.keys, xi);
+            const BlockWords w = block_words(pl, ((uint32_t)e.m0 >> 2) + (uint32_t)g, P.keys);
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
+            for (int p = 0; p < 2; ++p) {
                 if (M == 0) {
-                    prev = ph;
-                    if constexpr (is_pow_model(MODEL)) {
-                        ph = model.advance(ph, xi[q4], s2);
-                    } else {
-                        ph = model.step(ph, xi[q4]);
-                        s2 += xi[q4];
-                    }
-                    if constexpr (WALL) ph = real_min<Real>(ph, twouv - ph);
-                    const int step_index = e.m0 + 4 * g + q4;
-                    if (ph <= phi_end) {
-                        crossed = true;
-                        M = step_index + 1;
-                    } else if (step_index + 1 >= S.m_max) {
-                        M = step_index + 1;
-                    }
+                    const PairF64 np = pair_f64(p == 0 ? w.rad0 : w.rad1, p == 0 ? w.ang >> 16 : w.ang & 0xffffu);
+                    double last = ph;
+                    pair_steps_f64<MODEL, WALL>(model, np, twouv, ph, s2, [&](double x, int h) {
+                        prev = last;
+                        last = x;
+                        const int done = e.m0 + 4 * g + 2 * p + h + 1;
+                        crossed = x <= phi_end;
+                        if (crossed || done >= S.m_max) M = done;
+                        return M != 0;
+                    });
                 }
             }
             if (__all_sync(mask, M != 0)) break;
@@ -610,14 +648,12 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
 #define FPT_STEPPER_MAXNREG 64
 #endif
 //
-// KS: steps of a scheduling block.  FOLD (binary32): the sum of the normals is
-// folded into the running sum W every FOLD steps; that sets the rounding of ln w,
+// KS: steps of a scheduling block.  FOLD: the sum of the normals is folded into the running sum W every FOLD steps; that sets the rounding of ln w,
 // so it is what a caller's k_steps chooses, while the block length is free.
 template <typename Real, int PREC, int MODEL, bool WALL, int KS, int FOLD>
 __global__ void __maxnreg__(FPT_STEPPER_MAXNREG)
 stepper_kernel(const StepperParams P) {
-    static_assert(KS % (sizeof(Real) == 4 ? 16 : 4) == 0,
-                  "a scheduling block is a whole number of 16-step groups (binary32) or 4-step blocks (binary64)");
+    static_assert(KS % 16 == 0, "a scheduling block is a whole number of 16-step groups");
     using Entry = Pending<Real, PREC>;
     // dynamic shared memory: [set table][set starts][per-warp replay queues][parking slots]
     extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -743,26 +779,30 @@ stepper_kernel(const StepperParams P) {
             m += KS;
             event = live && !on;
         } else {
-            const uint32_t k0 = (uint32_t)m >> 2;
+            static_assert(KS == 16, "one Philox group per block");
+            bool on = true;
+            Reached64<MODEL> low;
+            low.reset(phi, phi_end);
+            pipelined_groups<KS>(pl, (uint32_t)m >> 4, P.keys, [&](const uint32_t* V, int j) {
 #pragma unroll
-            for (int g = 0; g < KS / 4; ++g) {
-                Real xi[4];
-                normals4<Real>(pl, k0 + (uint32_t)g, P.keys, xi);
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    if constexpr (is_pow_model(MODEL)) {
-                        phi = model.advance(phi, xi[q4], sblk);
-                    } else {
-                        phi = model.step(phi, xi[q4]);
-                        sblk += xi[q4];
-                    }
-                    if constexpr (WALL) phi = real_min<Real>(phi, twouv - phi);  // mirror at phi_uv
-                    mn = real_min<Real>(mn, phi);
-                }
-            }
+                for (int p = 0; p < 2; ++p)
+                    pair_steps_f64<MODEL, WALL>(model, group_pair_f64(V, j, p), twouv, phi, sblk, [&](double x, int) {
+                        low.see(x);
+                        return false;
+                    });
+                if ((4 * (j + 1)) % FOLD != 0) return;
+                // as above, every FOLD (4 or 8) steps
+                const int mg = m + 4 * (j + 1);
+                on = !low.any() && mg < m_max;
+                WSum<PREC> Wn = W;
+                Wn.add(sblk);
+                W.take(Wn, on);
+                sblk = 0.0;
+                phi0 = on ? phi : phi0;
+                m0 = on ? mg : m0;
+            });
             m += KS;
-            event = live && (mn <= phi_end || m >= m_max);
-            if (live && !event) W.add(sblk);
+            event = live && !on;
         }
         const unsigned ev = __ballot_sync(FULL, event);
         if (ev) {
@@ -802,7 +842,7 @@ stepper_kernel(const StepperParams P) {
                 park(v, 9 * stride, pl.r1_x1);
                 park(v, 10 * stride, pl.r1_set);
                 __syncwarp();
-                replay_batch<Real, PREC, MODEL, WALL, sizeof(Real) == 4 ? FOLD : KS>(q, 32, P, s_sets, lane, my_steps);
+                replay_batch<Real, PREC, MODEL, WALL, FOLD>(q, 32, P, s_sets, lane, my_steps);
                 __syncwarp();
                 const int rest = q_count - 32;
                 Entry tmp;
@@ -834,7 +874,7 @@ stepper_kernel(const StepperParams P) {
     }
     if (q_count > 0) {
         __syncwarp();
-        replay_batch<Real, PREC, MODEL, WALL, sizeof(Real) == 4 ? FOLD : KS>(q, q_count, P, s_sets, lane, my_steps);
+        replay_batch<Real, PREC, MODEL, WALL, FOLD>(q, q_count, P, s_sets, lane, my_steps);
     }
 
     // ---- total steps: warp reduce, one atomic per warp ----

@@ -1,24 +1,25 @@
 // Binary64 (reference) instantiations of the persistent stepper.  Built with
-// FMA contraction off (-fmad=false) so that every operation of the update is
-// rounded exactly as written, like the FP64 CPU definition it is checked
-// against.
+// FMA contraction off (-fmad=false) so that every operation is rounded exactly
+// as written.
 #include "stepper.cuh"
 #include "stepper_launch.h"
 
 namespace fpt {
 namespace {
 
-template <int MODEL, bool WALL, int KS>
+constexpr int kBlock64 = 16;  // steps of a scheduling block, whatever k_steps folds
+
+template <int MODEL, bool WALL, int FOLD>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) + (size_t)(block / 32) * warp_smem_bytes<double, FPT_PREC_F64>();
-    stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS, KS><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, kBlock64, FOLD><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
-template <int MODEL, bool WALL, int KS>
+template <int MODEL, bool WALL, int FOLD>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, KS, KS>,
-                         warp_smem_bytes<double, FPT_PREC_F64>(), &launch<MODEL, WALL, KS>};
+    return StepperKernel{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, kBlock64, FOLD>,
+                         warp_smem_bytes<double, FPT_PREC_F64>(), &launch<MODEL, WALL, FOLD>};
 }
 
 template <int MODEL, bool WALL>

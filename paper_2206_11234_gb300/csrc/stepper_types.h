@@ -47,7 +47,16 @@ struct SetConst {
     // polynomial potential V = sum_k poly[k] phi^k: binary64 coefficients, and
     // binary32 coefficients of V and V' (f_dpoly[k] = (k + 1) poly[k + 1])
     double poly[FPT_POLY_TERMS];
-    float f_poly[FPT_POLY_TERMS], f_dpoly[FPT_POLY_TERMS];
+    union {
+        struct {
+            float f_poly[FPT_POLY_TERMS], f_dpoly[FPT_POLY_TERMS];
+        };
+        // binary64 quadratic constant-bias step in psi = phi / sqrt(2 dN): psi_in, psi_end,
+        // 2 psi_uv, b c m dN, c m sqrt(dN)
+        struct {
+            double d_psi_in, d_psi_end, d_psi_twouv, d_c1, d_c2;
+        };
+    };
 };
 
 // Bytes of the per-set table at the start of the stepper's dynamic shared

@@ -102,3 +102,33 @@ def test_low_degree_polynomial_is_the_general_one(nat, precision, c, phi_uv):
         nat.fpt_simulate(p, N.numel(), 4.0, 2.5, phi_uv, 1e-3, 0.6, 9, N, lw)
         out.append((N, lw))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+def test_binary64_normals_over_all_angles_and_table_entries(nat):
+    """2^19 binary64 normals (every 16-bit angle about four times, every entry of
+    the logarithm's table) against the oracle's library functions: a few units in
+    the last place, as for the smaller sample of test_gpu_parity."""
+    import torch
+    import oracle
+    nb = 1 << 17
+    z = torch.empty(4 * nb, dtype=torch.float64, device="cuda")
+    nat.fpt_normals(11, 5, 1, 0, nb, "f64", z)
+    ref = np.concatenate([oracle.normals4(11, 5, 1, k) for k in range(nb)])
+    assert np.max(np.abs(z.cpu().numpy() - ref) / np.maximum(np.abs(ref), 1e-3)) < 4e-15
+
+
+@pytest.mark.parametrize("ks", [4, 8])
+@pytest.mark.parametrize("n_max", [0.006, 0.03, 0.032, 0.034, 1.0])
+def test_binary64_caps_inside_a_block(nat, ks, n_max):
+    """Caps at and beside the 4-, 8- and 16-step edges of the binary64 stepper against the oracle, run by run."""
+    import oracle
+    dN, b = 2e-3, 0.5
+    s = W.SetSpec(phi_in=1.45, m=1.0, b=b, dN=dN, n_max=n_max, n_traj=3000, phi_uv=1.5)
+    N, lw = batch(nat, [s], "f64", k_steps=ks)
+    r = oracle.make_run(m=1.0, phi_in=1.45, phi_uv=1.5, dN=dN, b=b, n_max=n_max, seed=3)
+    No, lwo, so = oracle.simulate(r, 3000)
+    N, lw = N.cpu().numpy(), lw.cpu().numpy()
+    fin = np.isfinite(No)
+    assert np.array_equal(np.isfinite(N), fin)
+    assert np.all(np.abs(N[fin] - No[fin]) <= 1e-12 * np.maximum(No[fin], dN))
+    assert np.all(np.abs(lw - lwo) <= 1e-12 * np.maximum(1.0, so * b * math.sqrt(dN)))
