@@ -13,6 +13,7 @@ The binding loads it instead of the default library when the environment
 variable FPT_DEBUG_LIB is 1.
 """
 import concurrent.futures as cf
+import math
 import os
 import shutil
 import struct
@@ -108,6 +109,30 @@ def f64_tables() -> str:
             % (pairs(trig), pairs(log), ",".join(word(2 * n * ln2 / one) for n in range(33))))
 
 
+def exp_table() -> str:
+    """The exponential's table of csrc/histogram.cu: 2^(j/4096), rounded correctly,
+    and ln 2 / 4096 as a 30-bit head and a binary64 tail."""
+    bits = 200
+    one = 1 << bits
+    root = 2 * one
+    for _ in range(12):
+        root = math.isqrt(root * one)
+    ln2, t, k = 0, 2 * one // 3, 1  # 2 atanh(1/3)
+    while t:
+        ln2 += t // k
+        t //= 9
+        k += 2
+    step = ln2 >> 12
+    head = step >> (bits - 42) << (bits - 42)  # step ~ 2^-12.5: 30 bits
+    x, table = one, []
+    for _ in range(1 << 12):
+        table.append((x / one).hex())
+        x = x * root >> bits
+    return ("__device__ const double kExp64[4096] = {%s};\nconstexpr double kExpStepHi = %s, kExpStepLo = %s, "
+            "kExpPerStep = %s;\n" % (",".join(table), (head / one).hex(), ((step - head) / one).hex(),
+                                     (one / step).hex()))
+
+
 def nvcc() -> str:
     for cand in (os.environ.get("NVCC"), shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
         if cand and os.path.exists(cand):
@@ -145,6 +170,8 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     os.makedirs(build_dir, exist_ok=True)
     with open(os.path.join(build_dir, "f64_tables.inc"), "w") as f:
         f.write(f64_tables())
+    with open(os.path.join(build_dir, "exp_table.inc"), "w") as f:
+        f.write(exp_table())
     cc = nvcc()
     extra = ["-DFPT_DEBUG=1"] if debug else []
 

@@ -372,16 +372,8 @@ int prepare(const fpt_params* p, const fpt_set* sets, int n_sets, bool with_hist
         if (with_hist) {
             rc = check_hist(sets[i].n_bins, sets[i].hist_lo, sets[i].hist_hi, 1);
             if (rc) return rc;
-            HistSeg h;
-            h.first = (long long)P->n_total;
-            h.n = sets[i].n_traj;
-            h.id_offset = sets[i].traj_offset;
-            h.lo = sets[i].hist_lo;
-            h.hi = sets[i].hist_hi;
-            h.d = (h.hi - h.lo) / (double)sets[i].n_bins;
-            h.n_bins = sets[i].n_bins;
-            h.n_sub = 1;
-            h.bin0 = P->total_bins;
+            const HistSeg h = hist_seg((long long)P->n_total, sets[i].n_traj, sets[i].traj_offset, sets[i].hist_lo,
+                                       sets[i].hist_hi, sets[i].n_bins, 1, P->total_bins);
             P->segs.push_back(h);
             P->total_bins += sets[i].n_bins;
             if (sets[i].n_bins > P->max_nb) P->max_nb = sets[i].n_bins;
@@ -520,7 +512,7 @@ void workspace_layout(const Prepared& P, WorkspaceLayout* L) {
     L->off_segs = align_up(L->off_sets + P.sets.size() * sizeof(SetConst), 256);
     L->bytes = align_up(L->off_segs + P.segs.size() * sizeof(HistSeg), 256);
     L->off_bin_idx = L->bytes;
-    L->total = P.segs.empty() ? L->bytes : L->bytes + align_up((size_t)P.n_total * sizeof(int), 256);
+    L->total = P.segs.empty() ? L->bytes : L->bytes + align_up((size_t)P.n_total * sizeof(uint16_t), 256);
 }
 
 void workspace_image(const Prepared& P, const WorkspaceLayout& L, std::vector<unsigned char>* img) {
@@ -562,7 +554,7 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
         rc = device_sm_count(&n_sm);
         if (rc) return rc;
         unsigned* status = reinterpret_cast<unsigned*>(ws + L.off_scratch + offsetof(StepperScratch, status));
-        int* bin_idx = L.total > L.bytes ? reinterpret_cast<int*>(ws + L.off_bin_idx) : nullptr;
+        uint16_t* bin_idx = L.total > L.bytes ? reinterpret_cast<uint16_t*>(ws + L.off_bin_idx) : nullptr;
         cudaError_t e = hist_launch(reinterpret_cast<const HistSeg*>(ws + L.off_segs), (int)P.segs.size(),
                                     P.max_nb, P.max_n, out_N, out_logw, bins, counts, n_sm, stream, status,
                                     bin_idx);
@@ -662,18 +654,9 @@ int fpt_histogram(const double* N, const double* logw, int64_t n, int32_t n_bins
     if (rc) return rc;
     if (!bins || !counts || (n > 0 && (!N || !logw))) return fail(FPT_EINVAL, "pointer is NULL");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    HistSeg h;
-    h.first = 0;
-    h.n = n;
-    h.id_offset = id_offset;
-    h.lo = lo;
-    h.hi = hi;
-    h.d = (hi - lo) / (double)n_bins;
-    h.n_bins = n_bins;
-    h.n_sub = n_sub;
-    h.bin0 = 0;
+    const HistSeg h = hist_seg(0, n, id_offset, lo, hi, n_bins, n_sub, 0);
     // workspace: the segment, then the status word (zero), then (not uploaded)
-    // one int per record for the bin index of pass 1
+    // one 16-bit word per record for the bin index of pass 1
     struct HistWork {
         HistSeg seg;
         unsigned status;
@@ -681,9 +664,9 @@ int fpt_histogram(const double* N, const double* logw, int64_t n, int32_t n_bins
     hw.seg = h;
     const size_t off_idx = align_up(sizeof(HistWork), 256);
     HistWork* d_w = nullptr;
-    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_w), off_idx + (size_t)n * sizeof(int), st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_w), off_idx + (size_t)n * sizeof(uint16_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "histogram workspace");
-    int* bin_idx = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(d_w) + off_idx);
+    uint16_t* bin_idx = reinterpret_cast<uint16_t*>(reinterpret_cast<unsigned char*>(d_w) + off_idx);
     e = cudaMemcpyAsync(d_w, &hw, sizeof(HistWork), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) rc = cuda_fail(e, "histogram upload");
     int n_sm = 0;

@@ -66,7 +66,7 @@ struct Prepared {
 
 // bytes: the part uploaded from the host image (scratch, set table, histogram
 // segments); total: bytes plus, with histograms, a region that is not
-// uploaded: one int per record (the bin index of histogram pass 1).
+// uploaded: one 16-bit word per record (the bin index of histogram pass 1).
 struct WorkspaceLayout {
     size_t off_scratch, off_sets, off_segs, bytes;
     size_t off_bin_idx, total;

@@ -4,20 +4,24 @@
 // Per bin: n_j, max ln w and, with x = ln w - max <= 0, s1 = sum exp(x),
 // s2 = sum exp(2 x), l_k = sum x^k for k = 1..4 (the moments of ln w behind the
 // lognormal estimator and normality test of §2.4).  Two streaming passes over the
-// records (HBM-resident; the passes are bound by the binary64 arithmetic, not
-// by the bytes):
-//   pass 1: classify each record (16 B read), per-bin max of ln w (shared-memory
-//           atomicMax on an order-preserving 64-bit key, one global atomic per bin
-//           and block); with a bin-index buffer, store each record's bin (4 B);
-//   pass 2: read ln w and the stored bin (or classify again without the buffer),
-//           max-shifted sums into shared-memory bins, lanes of a warp that hit
-//           the same bin (__match_any_sync) combined by their lowest lane, one
-//           peer per shuffle round, before one shared atomic per bin and warp.
+// records.  What bounds them is GB300's binary64 pipe, one warp instruction per SM
+// every 16 cycles whatever its active lanes, so both are written to spend few:
+//   pass 1: classify each record (16 B read) with one multiply-add, store its bin
+//           (2 B), keep the per-bin maximum of ln w as an order-preserving 64-bit
+//           key in shared memory (one global atomic per bin and block);
+//   pass 2: each block sorts a tile of ln w by bin in shared memory (counting sort,
+//           integers only), so that a thread adds up consecutive records of one
+//           bin in registers: 16 binary64 instructions per record, and sums leave
+//           for global memory once per bin change.
 // Bins are right-closed: j = ceil((N - lo)/d) - 1, clamped to [0, n_bins).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 
+#include "exp_table.inc"  // kExp64[4096] = 2^(j/4096), kExpStepHi + kExpStepLo = ln 2 / 4096, kExpPerStep its inverse
 #include "histogram.h"
 
 namespace fpt {
@@ -33,26 +37,42 @@ __device__ __forceinline__ double ord_value(unsigned long long k) {
 }
 
 constexpr unsigned long long kKeyNegInf = 0x000fffffffffffffull;  // ord_key(-inf)
-constexpr int kSums = 6;  // s1, s2, l1 .. l4 per bin
+constexpr int kSums = 6;                                          // s1, s2, l1 .. l4 per bin
+constexpr unsigned kNoBin = 0xffffu;
 
-// 0: in range (bin set), 1: N <= lo, 2: finite N > hi, 3: N not finite
-__device__ __forceinline__ int classify(double N, const HistSeg& h, unsigned long long gid, int& bin,
-                                        unsigned* status) {
-    if (!(N < __longlong_as_double(0x7ff0000000000000ll))) return 3;
-    if (N <= h.lo) return 1;
-    if (N > h.hi) return 2;
-    long long j = (long long)ceil((N - h.lo) / h.d) - 1;
+// Signed integers in the order of the numbers: NaN above +inf or below -inf by its sign.
+__host__ __device__ __forceinline__ long long signed_key(long long u) {
+    return u ^ (long long)((unsigned long long)(u >> 63) >> 1);
+}
+constexpr long long kSignedPosInf = 0x7ff0000000000000ll;
+constexpr long long kSignedNegInf = (long long)0x800fffffffffffffull;
+
+// Fixed point of the bin coordinate: N / d - lo / d + kFix has an ulp of 2^-36.
+constexpr double kFix = 98304.0;  // 1.5 x 2^16
+// largest |edge| / d for which the multiply-add is within 2 ulp (2^-35) of (N - lo) / d
+constexpr double kFastCoord = 8192.0;
+
+// Bin of N within its histogram; the comparisons are on integers and the
+// quotient is one multiply-add in fixed point.  Only where that lies within 4 ulp
+// of an edge does the division decide, as written.
+__device__ __forceinline__ int bin_of(double N, const HistSeg& h, unsigned* status) {
+    const double t = __fma_rn(N, h.inv_d, h.fix);
+    const unsigned hi = (unsigned)__double2hiint(t), lo4 = (unsigned)__double2loint(t) + 4u;
+    int j = (int)((hi >> 4) & 0x7fffu);
+    if (((hi + (lo4 < 4u ? 1u : 0u)) & 15u) == 0u && lo4 < 8u) {
+        const long long e = (long long)ceil((N - h.lo) / h.d) - 1;
 #if FPT_DEBUG
-    // rounding at the edges gives -1 or n_bins, which the clamp absorbs; more is a broken segment
-    if ((j < -1 || j > h.n_bins) && status) atomicOr(status, kStatusHistBin);
+        // rounding at the edges gives -1 or n_bins, which the clamp absorbs; more is a broken segment
+        if ((e < -1 || e > h.n_bins) && status) atomicOr(status, kStatusHistBin);
+#endif
+        j = e < 0 ? 0 : (int)(e < (long long)h.n_bins ? e : (long long)h.n_bins - 1);
+    }
+#if FPT_DEBUG
+    if (j >= h.n_bins && status) atomicOr(status, kStatusHistBin);
 #else
     (void)status;
 #endif
-    if (j < 0) j = 0;
-    if (j > h.n_bins - 1) j = h.n_bins - 1;
-    const int sub = (int)(gid % (unsigned long long)h.n_sub);
-    bin = sub * h.n_bins + (int)j;
-    return 0;
+    return j < h.n_bins ? j : h.n_bins - 1;
 }
 
 __global__ void hist_init(const HistSeg* __restrict__ segs, int n_segs, fpt_bin* __restrict__ bins,
@@ -78,134 +98,216 @@ __global__ void hist_init(const HistSeg* __restrict__ segs, int n_segs, fpt_bin*
     }
 }
 
-__global__ void hist_pass_max(const double* __restrict__ N, const double* __restrict__ lw,
-                              const HistSeg* __restrict__ segs, fpt_bin* __restrict__ bins,
-                              fpt_hist_counts* __restrict__ counts, unsigned* status,
-                              int* __restrict__ bin_idx) {
+constexpr int kMaxThreads = 512;  // pass 1
+constexpr int kMaxUnroll = 4;     // records of a thread in flight
+
+__global__ void __launch_bounds__(kMaxThreads) hist_pass_max(const double* __restrict__ N,
+                                                             const double* __restrict__ lw,
+                                                             const HistSeg* __restrict__ segs,
+                                                             fpt_bin* __restrict__ bins,
+                                                             fpt_hist_counts* __restrict__ counts, unsigned* status,
+                                                             uint16_t* __restrict__ bin_idx) {
     extern __shared__ unsigned long long s_key[];
     const HistSeg h = segs[blockIdx.y];
     const int nb = h.n_bins * h.n_sub;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) s_key[b] = kKeyNegInf;
     __syncthreads();
-    unsigned long long under = 0, over = 0, cens = 0;
-    const unsigned lane = threadIdx.x & 31u;
+    unsigned under = 0, over = 0, cens = 0;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    // warp-uniform loop: every lane of a warp runs the same iterations
-    for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < h.n;
-         base += stride) {
-        const long long i = base + lane;
-        int bin = -1;
-        unsigned long long key = 0;
-        if (i < h.n) {
-            const long long r = h.first + i;
-            const int cat = classify(N[r], h, h.id_offset + (unsigned long long)i, bin, status);
-            under += (cat == 1);
-            over += (cat == 2);
-            cens += (cat == 3);
-            if (cat == 0) key = ord_key(lw[r]);
-            if (bin_idx) bin_idx[r] = bin;
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    // jackknife subset of the thread's next record: ids advance by the stride
+    unsigned sub = 0, sub_step = 0;
+    if (h.n_sub > 1) {
+        sub = (unsigned)((h.id_offset + (unsigned long long)first) % (unsigned long long)h.n_sub);
+        sub_step = (unsigned)(stride % h.n_sub);
+    }
+    for (long long i = first; i < h.n; i += kMaxUnroll * stride) {
+        double x[kMaxUnroll], y[kMaxUnroll];
+#pragma unroll
+        for (int k = 0; k < kMaxUnroll; ++k)
+            if (i + k * stride < h.n) {
+                x[k] = N[h.first + i + k * stride];
+                y[k] = lw[h.first + i + k * stride];
+            }
+#pragma unroll
+        for (int k = 0; k < kMaxUnroll; ++k) {
+            if (i + k * stride >= h.n) break;
+            const long long s = signed_key(__double_as_longlong(x[k]));
+            unsigned bin = kNoBin;
+            if (s > h.key_hi) {
+                if (s < kSignedPosInf) ++over; else ++cens;
+            } else if (s <= h.key_lo) {
+                if (s >= kSignedNegInf) ++under; else ++cens;
+            } else {
+                bin = sub * (unsigned)h.n_bins + (unsigned)bin_of(x[k], h, status);
+                const unsigned long long key = ord_key(y[k]);
+                // rarely larger than what is there already
+                if (key > *reinterpret_cast<volatile unsigned long long*>(&s_key[bin])) atomicMax(&s_key[bin], key);
+            }
+            bin_idx[h.first + i + k * stride] = (uint16_t)bin;
+            sub += sub_step;
+            if (sub >= (unsigned)h.n_sub) sub -= (unsigned)h.n_sub;
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        // the group leader (lowest lane of the bin) takes the max over its peers,
-        // one peer per round: as many rounds as the largest group has members - 1
-        const bool leader = (int)lane == __ffs(peers) - 1;
-        unsigned rem = (leader && bin >= 0) ? (peers & ~(1u << lane)) : 0u;
-        unsigned long long best = key;
-        while (__any_sync(0xffffffffu, rem != 0u)) {
-            const int src = rem ? __ffs(rem) - 1 : (int)lane;
-            const unsigned long long v = __shfl_sync(0xffffffffu, key, src);
-            if (rem) best = v > best ? v : best;
-            rem &= rem - 1u;
-        }
-        if (bin >= 0 && leader) atomicMax(&s_key[bin], best);
     }
     __syncthreads();
     for (int b = threadIdx.x; b < nb; b += blockDim.x)
         if (s_key[b] != kKeyNegInf)
             atomicMax(reinterpret_cast<unsigned long long*>(&bins[h.bin0 + b].max_lw), s_key[b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        under += __shfl_xor_sync(0xffffffffu, under, o);
-        over += __shfl_xor_sync(0xffffffffu, over, o);
-        cens += __shfl_xor_sync(0xffffffffu, cens, o);
-    }
-    if (lane == 0 && (under | over | cens)) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].under), under);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].over), over);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].censored), cens);
+    under = __reduce_add_sync(0xffffffffu, under);
+    over = __reduce_add_sync(0xffffffffu, over);
+    cens = __reduce_add_sync(0xffffffffu, cens);
+    if ((threadIdx.x & 31u) == 0u) {
+        if (under) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].under), (unsigned long long)under);
+        if (over) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].over), (unsigned long long)over);
+        if (cens) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[blockIdx.y].censored), (unsigned long long)cens);
     }
 }
 
-__global__ void hist_pass_sum(const double* __restrict__ N, const double* __restrict__ lw,
-                              const HistSeg* __restrict__ segs, fpt_bin* __restrict__ bins, unsigned* status,
-                              const int* __restrict__ bin_idx) {
-    extern __shared__ double s_acc[];  // [nb][kSums] sums, then [nb] counts
+// exp(x) for x <= 0 in 8 binary64 instructions: x = k ln 2 / 4096 + r, the table's
+// 2^(k/4096) times the series of exp(r) to r^3, |r| <= 8.5e-5 (table-driven
+// exponential, Tang, ACM TOMS 15 (1989)); within about one unit in the last place.
+// Below -700, infinities and NaN: the library's.
+__device__ __forceinline__ double exp_neg(double x) {
+    if (((unsigned)__double2hiint(x) & 0x7fffffffu) > 0x4085e000u) return exp(x);
+    constexpr double kRound = 6755399441055744.0;  // 1.5 x 2^52
+    const double t = __fma_rn(x, kExpPerStep, kRound);
+    const int k = __double2loint(t);
+    const double kd = __dsub_rn(t, kRound);
+    const double r = __fma_rn(kd, -kExpStepLo, __fma_rn(kd, -kExpStepHi, x));
+    const double p = __fma_rn(__dmul_rn(r, r), __fma_rn(r, 1.0 / 6.0, 0.5), r);
+    const double T = __ldg(&kExp64[k & 4095]);
+    const double e = __fma_rn(T, p, T);
+    return __hiloint2double(__double2hiint(e) + (k >> 12) * (1 << 20), __double2loint(e));
+}
+
+constexpr int kSumThreads = 256;  // pass 2
+
+// Shared memory of pass 2: R records per thread sorted by bin (one padding element
+// per thread, so that threads reading their own runs do not collide), and a counter
+// per bin.
+template <int R>
+constexpr size_t sum_smem_bytes(int max_nb) {
+    return (size_t)kSumThreads * (R + 1) * (sizeof(double) + sizeof(uint16_t)) + (size_t)(max_nb + 1) * sizeof(int);
+}
+
+__device__ __forceinline__ void add_sums(fpt_bin* o, const double v[kSums]) {
+    atomicAdd(&o->s1, v[0]);
+    atomicAdd(&o->s2, v[1]);
+    atomicAdd(&o->l1, v[2]);
+    atomicAdd(&o->l2, v[3]);
+    atomicAdd(&o->l3, v[4]);
+    atomicAdd(&o->l4, v[5]);
+}
+
+template <int R>
+__global__ void __launch_bounds__(kSumThreads) hist_pass_sum(const double* __restrict__ lw,
+                                                             const HistSeg* __restrict__ segs,
+                                                             fpt_bin* __restrict__ bins,
+                                                             const uint16_t* __restrict__ bin_idx) {
+    constexpr int kTile = kSumThreads * R;
+    extern __shared__ double s_x[];
+    uint16_t* s_bin = reinterpret_cast<uint16_t*>(s_x + kSumThreads * (R + 1));
+    int* s_at = reinterpret_cast<int*>(s_bin + kSumThreads * (R + 1));  // count, then first place of a bin
+    __shared__ int s_warp[kSumThreads / 32];
     const HistSeg h = segs[blockIdx.y];
     const int nb = h.n_bins * h.n_sub;
-    unsigned long long* s_cnt = reinterpret_cast<unsigned long long*>(s_acc + kSums * nb);
-    for (int b = threadIdx.x; b < kSums * nb; b += blockDim.x) s_acc[b] = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) s_cnt[b] = 0ull;
-    __syncthreads();
-    const unsigned lane = threadIdx.x & 31u;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < h.n;
-         base += stride) {
-        const long long i = base + lane;
-        int bin = -1;
-        double v[kSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        if (i < h.n) {
-            const long long r = h.first + i;
-            if (bin_idx)
-                bin = bin_idx[r];
-            else if (classify(N[r], h, h.id_offset + (unsigned long long)i, bin, status) != 0)
-                bin = -1;
-            if (bin >= 0) {
-                const unsigned long long k =
-                    (unsigned long long)__double_as_longlong(bins[h.bin0 + bin].max_lw);
-                const double x = lw[r] - ord_value(k);
-                const double e = exp(x), x2 = x * x;
-                v[0] = e;
-                v[1] = e * e;
-                v[2] = x;
-                v[3] = x2;
-                v[4] = x2 * x;
-                v[5] = x2 * x2;
+    const unsigned FULL = 0xffffffffu;
+    const unsigned tid = threadIdx.x, lane = tid & 31u;
+    fpt_bin* out = bins + h.bin0;
+    for (long long base = (long long)blockIdx.x * kTile; base < h.n; base += (long long)gridDim.x * kTile) {
+        for (int b = tid; b < nb; b += kSumThreads) s_at[b] = 0;
+        __syncthreads();
+        // count the tile's records per bin; a record's rank among its bin's packed with the bin
+        double x[R];
+        unsigned at[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const long long i = base + k * kSumThreads + tid;
+            at[k] = kNoBin;
+            if (i < h.n) {
+                at[k] = bin_idx[h.first + i];
+                x[k] = lw[h.first + i];
             }
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        // the group leader sums its peers' values, one peer per round (no
-        // rounds when every lane of the warp has a bin of its own)
-        const bool leader = (int)lane == __ffs(peers) - 1;
-        unsigned rem = (leader && bin >= 0) ? (peers & ~(1u << lane)) : 0u;
-        double acc[kSums];
 #pragma unroll
-        for (int f = 0; f < kSums; ++f) acc[f] = v[f];
-        while (__any_sync(0xffffffffu, rem != 0u)) {
-            const int src = rem ? __ffs(rem) - 1 : (int)lane;
+        for (int k = 0; k < R; ++k)
+            if (at[k] != kNoBin) at[k] |= (unsigned)atomicAdd(&s_at[at[k]], 1) << 16;
+        __syncthreads();
+        // first places (exclusive sums of the counts); the counts go to the output here
+        int carry = 0;
+        for (int b0 = 0; b0 < nb; b0 += kSumThreads) {
+            const int b = b0 + (int)tid;
+            const int c = b < nb ? s_at[b] : 0;
+            int v = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(FULL, v, o);
+                if ((int)lane >= o) v += u;
+            }
+            if (lane == 31u) s_warp[tid >> 5] = v;
+            __syncthreads();
+            int before = carry;
+#pragma unroll
+            for (int w = 0; w < kSumThreads / 32; ++w) {
+                if (w < (int)(tid >> 5)) before += s_warp[w];
+                carry += s_warp[w];
+            }
+            if (b < nb) {
+                s_at[b] = before + v - c;
+                if (c) atomicAdd(reinterpret_cast<unsigned long long*>(&out[b].count), (unsigned long long)c);
+            }
+            __syncthreads();
+        }
+        const int total = carry;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const unsigned b = at[k] & 0xffffu;
+            if (b != kNoBin) {
+                const int p = s_at[b] + (int)(at[k] >> 16);
+                s_x[p + p / R] = x[k];
+                s_bin[p + p / R] = (uint16_t)b;
+            }
+        }
+        __syncthreads();
+        // every thread's R consecutive places: one bin after the other
+        double v[kSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        unsigned cur = kNoBin;
+        double mx = 0.0;
+        const int mine = min(R, total - (int)tid * R);
+        for (int k = 0; k < mine; ++k) {
+            const unsigned b = s_bin[tid * (R + 1) + k];
+            if (b != cur) {
+                if (cur != kNoBin) add_sums(&out[cur], v);
+#pragma unroll
+                for (int f = 0; f < kSums; ++f) v[f] = 0.0;
+                cur = b;
+                mx = ord_value((unsigned long long)__double_as_longlong(out[b].max_lw));
+            }
+            const double y = __dsub_rn(s_x[tid * (R + 1) + k], mx);
+            const double e = exp_neg(y), y2 = __dmul_rn(y, y);
+            v[0] = __dadd_rn(v[0], e);
+            v[1] = __fma_rn(e, e, v[1]);
+            v[2] = __dadd_rn(v[2], y);
+            v[3] = __dadd_rn(v[3], y2);
+            v[4] = __fma_rn(y2, y, v[4]);
+            v[5] = __fma_rn(y2, y2, v[5]);
+        }
+        // the last bins of a warp's threads: lanes of one bin are neighbours; add
+        // up each group towards its highest lane, which writes it
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned cb = __shfl_up_sync(FULL, cur, o);
+            const bool same = (int)lane >= o && cb == cur && cur != kNoBin;
+            if (!__any_sync(FULL, same)) break;
 #pragma unroll
             for (int f = 0; f < kSums; ++f) {
-                const double y = __shfl_sync(0xffffffffu, v[f], src);
-                if (rem) acc[f] += y;
+                const double u = __shfl_up_sync(FULL, v[f], o);
+                if (same) v[f] = __dadd_rn(v[f], u);
             }
-            rem &= rem - 1u;
         }
-        if (bin >= 0 && leader) {
-#pragma unroll
-            for (int f = 0; f < kSums; ++f) atomicAdd(&s_acc[kSums * bin + f], acc[f]);
-            atomicAdd(&s_cnt[bin], (unsigned long long)__popc(peers));
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        if (s_cnt[b] == 0ull) continue;
-        fpt_bin* o = bins + h.bin0 + b;
-        atomicAdd(&o->s1, s_acc[kSums * b + 0]);
-        atomicAdd(&o->s2, s_acc[kSums * b + 1]);
-        atomicAdd(&o->l1, s_acc[kSums * b + 2]);
-        atomicAdd(&o->l2, s_acc[kSums * b + 3]);
-        atomicAdd(&o->l3, s_acc[kSums * b + 4]);
-        atomicAdd(&o->l4, s_acc[kSums * b + 5]);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&o->count), s_cnt[b]);
+        const unsigned next = __shfl_down_sync(FULL, cur, 1);
+        if (cur != kNoBin && (lane == 31u || next != cur)) add_sums(&out[cur], v);
+        __syncthreads();
     }
 }
 
@@ -218,38 +320,80 @@ __global__ void hist_final(const HistSeg* __restrict__ segs, fpt_bin* __restrict
     }
 }
 
+template <int R>
+cudaError_t launch_sum(const HistSeg* d_segs, int n_segs, int max_nb, long long max_n, const double* lw, fpt_bin* bins,
+                       int n_sm, cudaStream_t stream, const uint16_t* bin_idx) {
+    cudaError_t e = cudaFuncSetAttribute(hist_pass_sum<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sum_smem_bytes<R>(FPT_MAX_HIST_BINS));
+    if (e != cudaSuccess) return e;
+    const size_t smem = sum_smem_bytes<R>(max_nb);
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hist_pass_sum<R>, kSumThreads, smem);
+    if (e != cudaSuccess) return e;
+    const long long tiles = std::max(1LL, (max_n + kSumThreads * R - 1) / (kSumThreads * R));
+    const long long cap = std::max(1LL, ((long long)std::max(per_sm, 1) * n_sm + n_segs - 1) / n_segs);
+    hist_pass_sum<R><<<dim3((unsigned)std::min(tiles, cap), n_segs), kSumThreads, smem, stream>>>(lw, d_segs, bins,
+                                                                                                 bin_idx);
+    return cudaGetLastError();
+}
+
+long long host_key(double x) {
+    x += 0.0;  // -0 compares like +0
+    long long u;
+    std::memcpy(&u, &x, sizeof(u));
+    return signed_key(u);
+}
+
 }  // namespace
 
-size_t hist_smem_bytes(int max_nb) { return (size_t)max_nb * (kSums * sizeof(double) + 8); }
+HistSeg hist_seg(long long first, long long n, unsigned long long id_offset, double lo, double hi, int n_bins,
+                 int n_sub, long long bin0) {
+    HistSeg h;
+    h.first = first;
+    h.n = n;
+    h.id_offset = id_offset;
+    h.lo = lo;
+    h.hi = hi;
+    h.d = (hi - lo) / (double)n_bins;
+    h.n_bins = n_bins;
+    h.n_sub = n_sub;
+    h.bin0 = bin0;
+    h.key_lo = host_key(lo);
+    h.key_hi = host_key(hi);
+    // outside the fixed point's range every record takes the division
+    h.inv_d = 1.0 / h.d;
+    const bool fast = std::isnormal(h.d) && std::isnormal(h.inv_d) && std::fabs(lo) * h.inv_d <= kFastCoord &&
+                      std::fabs(hi) * h.inv_d <= kFastCoord;
+    if (!fast) h.inv_d = 0.0;
+    h.fix = kFix - lo * h.inv_d;
+    return h;
+}
 
 cudaError_t hist_launch(const HistSeg* d_segs, int n_segs, int max_nb, long long max_n,
                         const double* N, const double* lw, fpt_bin* bins, fpt_hist_counts* counts,
-                        int n_sm, cudaStream_t stream, unsigned* status, int* bin_idx) {
-    const size_t smem_sum = hist_smem_bytes(max_nb);
+                        int n_sm, cudaStream_t stream, unsigned* status, uint16_t* bin_idx) {
     const size_t smem_max = (size_t)max_nb * sizeof(unsigned long long);
-    // opt in to large dynamic shared memory (per device; cheap to repeat)
-    cudaError_t e = cudaFuncSetAttribute(hist_pass_sum, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)hist_smem_bytes(FPT_MAX_HIST_BINS));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(hist_pass_max, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(FPT_MAX_HIST_BINS * sizeof(unsigned long long)));
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const int threads = 256;
     const int init_blocks = (max_nb + threads - 1) / threads;
     hist_init<<<dim3(init_blocks, n_segs), threads, 0, stream>>>(d_segs, n_segs, bins, counts);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // about two waves of blocks over all segments, at least one block per segment
-    long long want = (max_n + threads * 8 - 1) / (threads * 8);
-    int per_seg = (int)(want < 1 ? 1 : want);
-    const int cap = (2 * n_sm + n_segs - 1) / n_segs;
-    if (per_seg > cap) per_seg = cap < 1 ? 1 : cap;
-    hist_pass_max<<<dim3(per_seg, n_segs), threads, smem_max, stream>>>(N, lw, d_segs, bins, counts, status,
-                                                                        bin_idx);
+    // as many blocks as fit at once, at least one per segment
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hist_pass_max, kMaxThreads, smem_max);
+    if (e != cudaSuccess) return e;
+    const long long want = std::max(1LL, (max_n + kMaxThreads - 1) / kMaxThreads);
+    const long long cap = std::max(1LL, ((long long)std::max(per_sm, 1) * n_sm + n_segs - 1) / n_segs);
+    hist_pass_max<<<dim3((unsigned)std::min(want, cap), n_segs), kMaxThreads, smem_max, stream>>>(
+        N, lw, d_segs, bins, counts, status, bin_idx);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    hist_pass_sum<<<dim3(per_seg, n_segs), threads, smem_sum, stream>>>(N, lw, d_segs, bins, status, bin_idx);
-    e = cudaGetLastError();
+    // long runs per thread amortise the last bins' reduction, short ones spread small inputs over the SMs
+    if (max_n * n_segs >= 4LL * n_sm * kSumThreads * 32)
+        e = launch_sum<32>(d_segs, n_segs, max_nb, max_n, lw, bins, n_sm, stream, bin_idx);
+    else
+        e = launch_sum<8>(d_segs, n_segs, max_nb, max_n, lw, bins, n_sm, stream, bin_idx);
     if (e != cudaSuccess) return e;
     hist_final<<<dim3(init_blocks, n_segs), threads, 0, stream>>>(d_segs, bins);
     return cudaGetLastError();
