@@ -32,7 +32,8 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUD
 UNITS = {
     "abi.cu": [],
     "histogram.cu": [],
-    "stepper_f32.cu": [],
+    "stepper_f32_kahan.cu": [],
+    "stepper_f32_f64acc.cu": [],
     "stepper_pow.cu": [],
     "stepper_f64.cu": ["-fmad=false", "-DFPT_STEPPER_MAXNREG=128"],
     "rng_probe.cu": ["-fmad=false"],

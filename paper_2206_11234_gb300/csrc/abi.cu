@@ -9,8 +9,10 @@
 #include <atomic>
 #include <cstddef>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "abi_internal.h"
@@ -423,11 +425,43 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
     return FPT_OK;
 }
 
-// The grid of the persistent stepper: as many warps per SM as fit, fewer where
-// the launch would trail off.  A run's speed is inversely proportional to the
-// warps that share its SM, the SM's throughput hardly depends on them (16 warps
-// per SM run 2.5 % slower than 32 on the drift ladder, 24 warps 1 %), so the last
-// and longest runs finish sooner with fewer.  In units of an SM's time per
+// CTAs of a stepper that fit on one SM, by the occupancy API; kept per kernel and
+// shape (the answer is the kernel's alone), since a query costs a small call more
+// than a microsecond.
+static int stepper_ctas(const void* func, int block, size_t smem, int* per_sm) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t>, int> cache;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_tuple(dev, func, block, smem);
+    const auto it = cache.find(key);
+    if (it != cache.end()) {
+        *per_sm = it->second;
+        return FPT_OK;
+    }
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    if (e != cudaSuccess) return cuda_fail(e, "stepper shared memory");
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, func, block, smem);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    if (*per_sm < 1) *per_sm = 1;
+    if (cache.size() >= 4096) cache.clear();
+    cache[key] = *per_sm;
+    return FPT_OK;
+}
+
+// Time of a step, in cycles, when `warps` warps share a scheduler: a few are bound
+// by their own chains, more of them by the XU pipe and the issue slots (wall runs,
+// 1, 2, 3, 4, 8 warps: 65, 81, 108, 140, 260 cycles).
+static double step_cycles(double warps) { return std::fmax(49.0 + 16.0 * warps, 14.0 + 31.0 * warps); }
+
+// The launch shape of the persistent stepper; results do not depend on it.
+//
+// Resident warps.  A run's speed is inversely proportional to the warps that share
+// its SM, the SM's throughput hardly depends on them (16 warps per SM run 2.5 %
+// slower than 32 on the drift ladder, 24 warps 1 %), so where run lengths spread
+// the last and longest runs finish sooner with fewer.  In units of an SM's time per
 // warp-step, a full SM of r warps needs r x steps for one run's steps, and
 // total / (32 n_sm) for its share of the whole work; measured (us):
 //   tail / work                    16 warps   24 warps   32 warps
@@ -438,34 +472,37 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
 // The longest expected run bounds the launch as well (64 uneven sets of 4096:
 // 8020 us with 14 warps per SM, 11235 with 24).
 //
-// Threads per block (0: free): results do not depend on them.  The largest
-// block whose CTAs load every SM alike (40,000 runs are 157 CTAs of 256 threads,
-// two of them on five of the 152 SMs: 6.08 ms; as 128-thread CTAs 4.82 ms).
-int stepper_grid(const StepperKernel& k, int n_sets, unsigned long long n_total, const RunLengths& len, int* block,
-                 int* grid) {
+// Bench (binary32).  Runs of one length that are not a whole number of waves leave
+// some schedulers with one warp more than the others: 40,000 runs are 2.06 warps
+// per scheduler, and the launch takes the time of three.  Fewer warps that take
+// turns at a few more runs each (StepperParams::bench) even that out.
+//
+// Threads per block (0: free): the largest block whose CTAs load every SM alike
+// (40,000 runs are 157 CTAs of 256 threads, two of them on five of the 152 SMs:
+// 6.08 ms; as 128-thread CTAs 4.82 ms).
+int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsigned long long n_total,
+                 const RunLengths& len, LaunchShape* shape) {
     int n_sm = 0;
     int rc = device_sm_count(&n_sm);
     if (rc) return rc;
-    cudaError_t e = cudaFuncSetAttribute(k.func, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-    if (e != cudaSuccess) return cuda_fail(e, "stepper shared memory");
     const double share = len.total / (32.0 * n_sm);
-    const bool fixed = *block != 0;
-    int best = 0;
+    const int fixed = shape->block;
     // many runs: 256 threads (up to 1 % faster); fewer: 128 (3 x 45,000 equal runs 1652 us, 1774 with
     // 256; 64 uneven sets of 16,384 runs 26.8 ms, 30.0 with 256)
     const int first = n_total >= 32ull * kTrailingRuns ? 256 : 128;
-    for (int b = fixed ? *block : first; b >= 32; b >>= 1) {
-        const size_t smem = stepper_smem(k, b, n_sets);
+    const bool uneven = len.longest * (double)n_total > 1.5 * len.total;
+    int best = 0;
+    shape->bench = 0;
+    for (int b = fixed ? fixed : first; b >= 32; b >>= 1) {
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.func, b, smem);
-        if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+        rc = stepper_ctas(k.func, b, stepper_smem(k, b, n_sets, 0), &per_sm);
+        if (rc) return rc;
         const int warps = b / 32, full = per_sm * warps;
         int r = full;
         const double trail = share > 0.0 ? len.tail * full / share : 0.0;
         if (trail > 0.15) r = full / 2;
         else if (trail > 0.06) r = 3 * full / 4;
-        if (len.longest * (double)n_total > 1.5 * len.total)
-            r = std::min(r, std::max(8, (int)std::ceil(1.25 * share / len.longest)));
+        if (uneven) r = std::min(r, std::max(8, (int)std::ceil(1.25 * share / len.longest)));
         per_sm = std::max(1, r / warps);
         const unsigned long long need = std::max(1ull, (n_total + b - 1) / b);
         const unsigned long long room = (unsigned long long)per_sm * n_sm;
@@ -473,10 +510,38 @@ int stepper_grid(const StepperKernel& k, int n_sets, unsigned long long n_total,
         const int load = need <= room ? (int)((need + n_sm - 1) / n_sm) * warps : per_sm * warps;
         if (best == 0 || (need <= room && load < best)) {
             best = load;
-            *block = b;
-            *grid = (int)std::min(need, room);
+            shape->block = b;
+            shape->grid = (int)std::min(need, room);
         }
         if (fixed) break;
+    }
+    if (!k.bench_func || uneven || !(len.tail <= 0.1 * len.longest)) return FPT_OK;
+    const int b = fixed ? fixed : 128, warps = b / 32;
+    int per_sm = 0;
+    rc = stepper_ctas(k.bench_func, b, stepper_smem(k, b, n_sets, 32), &per_sm);
+    if (rc) return rc;
+    // waves of all warps that fit, and a rest: the time of a step of every run
+    const double x = (double)n_total / (128.0 * n_sm);  // warps per scheduler, if all ran at once
+    const double k_full = best / 4.0;
+    const double waves = std::floor(x / k_full + 1e-9);
+    double time = waves * step_cycles(k_full) + (x > waves * k_full ? step_cycles(std::ceil(x - waves * k_full)) : 0.0);
+    if (waves == 0.0) time = step_cycles(std::ceil(k_full));
+    time *= 0.95;  // what the turns cost
+    for (int c = per_sm; c >= 1; --c) {
+        const double kc = c * warps / 4.0, gens = std::floor(x / kc);
+        if (gens < 1.0) continue;
+        const double per_lane = x / (gens * kc);  // runs per lane and generation
+        const int bench = (int)std::ceil(32.0 * (per_lane - 1.0) - 1e-9);
+        if (bench < 1 || bench > 32) continue;
+        const double t = gens * (32.0 + bench) / 32.0 * step_cycles(kc);
+        if (t < time) {
+            time = t;
+            shape->block = b;
+            shape->grid = c * n_sm;
+            shape->bench = bench;
+            // some 32 turns in a run
+            shape->bench_every = std::min(64, std::max(4, (int)(len.longest / (64.0 * 32.0))));
+        }
     }
     return FPT_OK;
 }
@@ -527,10 +592,10 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
                 uint64_t seed, double* out_N, double* out_logw, fpt_bin* bins, fpt_hist_counts* counts,
                 cudaStream_t stream, const std::function<int()>& after_stepper) {
     StepperKernel k;
-    int block = 0, grid = 0;
-    int rc = pick_stepper(p, P.wall, &k, &block);
+    LaunchShape shape;
+    int rc = pick_stepper(p, P.wall, &k, &shape.block);
     if (rc) return rc;
-    rc = stepper_grid(k, (int)P.sets.size(), P.n_total, P.len, &block, &grid);
+    rc = stepper_grid(p, k, (int)P.sets.size(), P.n_total, P.len, &shape);
     if (rc) return rc;
     StepperParams a;
     a.keys = philox_keys(seed);
@@ -540,9 +605,11 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
     a.out_N = out_N;
     a.out_logw = out_logw;
     a.scratch = reinterpret_cast<StepperScratch*>(ws + L.off_scratch);
+    a.bench = shape.bench;
+    a.bench_every = shape.bench_every;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
     if (P.n_total > 0) {
-        cudaError_t e = k.launch(a, grid, block, stream);
+        cudaError_t e = (shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
         if (e != cudaSuccess) return cuda_fail(e, "stepper launch");
     }
     if (after_stepper) {

@@ -83,9 +83,13 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block);
 // Launch shape chosen by fpt_autotune for this device and kind of launch, if any.
 bool tuned_shape(int precision, int model, bool wall, int* block, int* ks);
 void clear_tuned_shapes();
-// Grid of a persistent launch, and its threads per block where *block is 0.
-int stepper_grid(const StepperKernel& k, int n_sets, unsigned long long n_total, const RunLengths& len, int* block,
-                 int* grid);
+struct LaunchShape {
+    int block = 0, grid = 0;  // block: 0 where stepper_grid may choose it
+    int bench = 0;            // runs that take turns with each warp's 32 ...
+    int bench_every = 0;      // ... every so many scheduling blocks
+};
+int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsigned long long n_total,
+                 const RunLengths& len, LaunchShape* shape);
 void workspace_layout(const Prepared& P, WorkspaceLayout* L);
 void workspace_image(const Prepared& P, const WorkspaceLayout& L, std::vector<unsigned char>* img);
 // Enqueues the stepper and, with bins, the histogram kernels on `stream`.

@@ -127,10 +127,10 @@ extern "C" int fpt_simulate_batch_noalloc(const fpt_params* p, const fpt_set* se
     if (!out_N || !out_logw) return fail(FPT_EINVAL, "output pointer is NULL");
 
     StepperKernel k;
-    int block = 0, grid = 0;
-    rc = pick_stepper(p, wall, &k, &block);
+    LaunchShape shape;
+    rc = pick_stepper(p, wall, &k, &shape.block);
     if (rc) return rc;
-    rc = stepper_grid(k, n_sets, n_total, len, &block, &grid);
+    rc = stepper_grid(p, k, n_sets, n_total, len, &shape);
     if (rc) return rc;
     unsigned char* ws = nullptr;
     rc = scratch_address(&ws);
@@ -150,8 +150,10 @@ extern "C" int fpt_simulate_batch_noalloc(const fpt_params* p, const fpt_set* se
     a.out_N = out_N;
     a.out_logw = out_logw;
     a.scratch = reinterpret_cast<StepperScratch*>(ws);
+    a.bench = shape.bench;
+    a.bench_every = shape.bench_every;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
-    e = k.launch(a, grid, block, stream);
+    e = (shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
     if (e != cudaSuccess) return cuda_fail(e, "stepper launch");
 
     StepperScratch host;

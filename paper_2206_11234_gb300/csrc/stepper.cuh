@@ -491,7 +491,6 @@ struct Pending {
 };
 
 constexpr int kQueueCap = 64;  // per warp: up to 31 waiting + 32 new
-constexpr int kParkWords = 12;  // per thread: a run's live state during a batch replay
 
 // Park / unpark 32-bit words through volatile shared memory, so the values are
 // really dead in registers while the replay runs (no store-to-load forwarding).
@@ -650,8 +649,10 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
 //
 // KS: steps of a scheduling block.  FOLD: the sum of the normals is folded into the running sum W every FOLD steps; that sets the rounding of ln w,
 // so it is what a caller's k_steps chooses, while the block length is free.
-template <typename Real, int PREC, int MODEL, bool WALL, int KS, int FOLD>
-__global__ void __maxnreg__(FPT_STEPPER_MAXNREG)
+// BENCH: with runs that take turns (StepperParams::bench); for at most 16 warps per
+// SM, so with twice the registers (at 64 the turns' state cost the step 4-14 %).
+template <typename Real, int PREC, int MODEL, bool WALL, int KS, int FOLD, bool BENCH = false>
+__global__ void __maxnreg__(BENCH ? 128 : FPT_STEPPER_MAXNREG)
 stepper_kernel(const StepperParams P) {
     static_assert(KS % 16 == 0, "a scheduling block is a whole number of 16-step groups");
     using Entry = Pending<Real, PREC>;
@@ -662,9 +663,12 @@ stepper_kernel(const StepperParams P) {
     long long* s_first = reinterpret_cast<long long*>(s_dyn + (size_t)n_sets * sizeof(SetConst));
     unsigned char* s_queue = s_dyn + stepper_table_bytes(n_sets);
     Entry* q = reinterpret_cast<Entry*>(s_queue) + (threadIdx.x >> 5) * kQueueCap;
-    // parking slots follow the queues: kParkWords words per thread, interleaved by thread
+    // parking slots follow the queues: kParkWords words per thread, interleaved by
+    // thread; then each warp's bench: kParkWords words per run, interleaved by run
     volatile unsigned* park_slot = reinterpret_cast<volatile unsigned*>(
         s_queue + (size_t)(blockDim.x >> 5) * kQueueCap * sizeof(Entry)) + threadIdx.x;
+    volatile unsigned* bench_slot = park_slot - threadIdx.x + blockDim.x * kParkWords +
+                                    (threadIdx.x >> 5) * (unsigned)(P.bench * kParkWords);
     for (int i = threadIdx.x; i < n_sets; i += blockDim.x) {
         s_sets[i] = P.sets[i];
         s_first[i] = P.sets[i].ticket0;
@@ -690,12 +694,90 @@ stepper_kernel(const StepperParams P) {
     unsigned long long my_steps = 0;
     int q_count = 0;  // warp-uniform
 
+    // a run's state to and from shared memory: word j at v[j * stride]
+    auto save = [&](volatile unsigned* v, int stride) {
+        park_r<Real>(v, 0 * stride, stride, phi);  // words 0, 1
+        park_w<PREC>(v, 2 * stride, stride, W);    // words 2, 3
+        park(v, 4 * stride, (unsigned)m);
+        park(v, 5 * stride, (unsigned)rec);
+        park(v, 6 * stride, (unsigned)(rec >> 32));
+        park(v, 7 * stride, (unsigned)set | (live ? 0x40000000u : 0u) | (exhausted ? 0x80000000u : 0u));
+        park(v, 8 * stride, pl.r1_x0);
+        park(v, 9 * stride, pl.r1_x1);
+        park(v, 10 * stride, pl.r1_set);
+    };
+    auto load = [&](volatile unsigned* v, int stride) {
+        phi = unpark_r<Real>(v, 0 * stride, stride);
+        unpark_w<PREC>(v, 2 * stride, stride, W);
+        m = (int)unpark(v, 4 * stride);
+        rec = (unsigned long long)unpark(v, 5 * stride) | ((unsigned long long)unpark(v, 6 * stride) << 32);
+        const unsigned sf = unpark(v, 7 * stride);
+        set = (int)(sf & 0x3fffffffu);
+        live = (sf & 0x40000000u) != 0u;
+        exhausted = (sf & 0x80000000u) != 0u;
+        pl.r1_x0 = unpark(v, 8 * stride);
+        pl.r1_x1 = unpark(v, 9 * stride);
+        pl.r1_set = unpark(v, 10 * stride);
+        const SetConst& S = s_sets[set];
+        model.load(S);
+        phi_end = set_phi_end<Real, MODEL>(S);
+        twouv = set_twouv<Real, MODEL>(S);
+        m_max = S.m_max;
+    };
+
+    // The bench: P.bench runs beside the warp's 32, filled once, before the lanes.
+    // Every P.bench_every blocks its runs change places with live lanes, in turn, so
+    // that all 32 + bench runs advance alike; when the tickets are gone, idle lanes
+    // take the bench's runs.
+    int waiting = 0;    // warp-uniform: runs on the bench
+    int until = 0;      // blocks to the next change
+    unsigned turn = 0;  // first lane of the next change
+    bool filling = BENCH;
+
     for (;;) {
+        // ---- a change of places ----
+        if constexpr (BENCH) {
+            if (waiting > 0 && --until < 0) {
+                until = P.bench_every;
+                const unsigned i = (lane - turn) & 31u;
+                turn += (unsigned)waiting;
+                if ((int)i < waiting && live) {
+                    // through the parking slot: the outgoing state is dead in registers before the load
+                    volatile unsigned* b = bench_slot + i;
+                    save(park_slot, (int)blockDim.x);
+                    load(b, P.bench);
+#pragma unroll
+                    for (int j = 0; j < kParkWords - 1; ++j) b[j * P.bench] = park_slot[j * (int)blockDim.x];
+                }
+                __syncwarp();
+            }
+        }
         // ---- refill: lanes without a run take tickets (one atomic per warp) ----
         for (;;) {
-            const bool want = !live && !exhausted;
+            const bool want = !live && !exhausted && !(BENCH && filling && (int)lane >= P.bench);
             const unsigned need = __ballot_sync(FULL, want);
-            if (need == 0u) break;
+            if (need == 0u) {
+                if constexpr (!BENCH) break;
+                if (filling) {
+                    // the bench's runs, not yet started, leave the lanes
+                    const unsigned on = __ballot_sync(FULL, live);
+                    if (live) save(bench_slot + __popc(on & lt_mask), P.bench);
+                    live = false;
+                    waiting = __popc(on);
+                    until = P.bench_every;
+                    filling = false;
+                    __syncwarp();
+                    continue;
+                }
+                const unsigned idle = __ballot_sync(FULL, !live);
+                if (idle != 0u && waiting > 0) {
+                    const int i = waiting - 1 - __popc(idle & lt_mask);
+                    if (!live && i >= 0) load(bench_slot + i, P.bench);
+                    waiting = max(0, waiting - __popc(idle));
+                    __syncwarp();
+                }
+                break;
+            }
             const int leader = __ffs(need) - 1;
             unsigned long long base = 0;
             if ((int)lane == leader) base = atomicAdd(&P.scratch->ticket, (unsigned long long)__popc(need));
@@ -830,17 +912,7 @@ stepper_kernel(const StepperParams P) {
 #endif
             if (q_count >= 32) {
                 // park this lane's run (the stride keeps one thread's words in one bank)
-                const int stride = (int)blockDim.x;
-                volatile unsigned* v = park_slot;
-                park_r<Real>(v, 0 * stride, stride, phi);  // words 0, 1
-                park_w<PREC>(v, 2 * stride, stride, W);    // words 2, 3
-                park(v, 4 * stride, (unsigned)m);
-                park(v, 5 * stride, (unsigned)rec);
-                park(v, 6 * stride, (unsigned)(rec >> 32));
-                park(v, 7 * stride, (unsigned)set | (live ? 0x40000000u : 0u) | (exhausted ? 0x80000000u : 0u));
-                park(v, 8 * stride, pl.r1_x0);
-                park(v, 9 * stride, pl.r1_x1);
-                park(v, 10 * stride, pl.r1_set);
+                save(park_slot, (int)blockDim.x);
                 __syncwarp();
                 replay_batch<Real, PREC, MODEL, WALL, FOLD>(q, 32, P, s_sets, lane, my_steps);
                 __syncwarp();
@@ -851,24 +923,7 @@ stepper_kernel(const StepperParams P) {
                 if ((int)lane < rest) q[lane] = tmp;
                 __syncwarp();
                 q_count = rest;
-                // unpark
-                phi = unpark_r<Real>(v, 0 * stride, stride);
-                unpark_w<PREC>(v, 2 * stride, stride, W);
-                m = (int)unpark(v, 4 * stride);
-                rec = (unsigned long long)unpark(v, 5 * stride) |
-                      ((unsigned long long)unpark(v, 6 * stride) << 32);
-                const unsigned sf = unpark(v, 7 * stride);
-                set = (int)(sf & 0x3fffffffu);
-                live = (sf & 0x40000000u) != 0u;
-                exhausted = (sf & 0x80000000u) != 0u;
-                pl.r1_x0 = unpark(v, 8 * stride);
-                pl.r1_x1 = unpark(v, 9 * stride);
-                pl.r1_set = unpark(v, 10 * stride);
-                const SetConst& S = s_sets[set];
-                model.load(S);
-                phi_end = set_phi_end<Real, MODEL>(S);
-                twouv = set_twouv<Real, MODEL>(S);
-                m_max = S.m_max;
+                load(park_slot, (int)blockDim.x);
             }
         }
     }

@@ -27,7 +27,7 @@ StepperKernel by_ks(int ks) {
     switch (ks) {
         case 4: return make<MODEL, WALL, 4>();
         case 8: return make<MODEL, WALL, 8>();
-        default: return StepperKernel{nullptr, 0, nullptr};
+        default: return StepperKernel{};
     }
 }
 
@@ -43,7 +43,7 @@ StepperKernel stepper_f64(int model, bool wall, int k_steps) {
     if (model == FPT_MODEL_CONSTANT) return by_wall<FPT_MODEL_CONSTANT>(wall, k_steps);
     if (model == FPT_MODEL_POLYNOMIAL) return by_wall<FPT_MODEL_POLYNOMIAL>(wall, k_steps);
     if (model == kModelPowReal) return by_wall<kModelPowReal>(wall, k_steps);
-    return StepperKernel{nullptr, 0, nullptr};
+    return StepperKernel{};
 }
 
 }  // namespace fpt

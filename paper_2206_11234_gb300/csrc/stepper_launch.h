@@ -8,13 +8,16 @@
 namespace fpt {
 
 struct StepperKernel {
-    const void* func;     // for occupancy queries; nullptr = no such instantiation
-    int warp_smem_bytes;  // dynamic shared memory per warp (replay queue + parking)
-    cudaError_t (*launch)(const StepperParams&, int grid, int block, cudaStream_t stream);
+    const void* func = nullptr;  // for occupancy queries; nullptr = no such instantiation
+    int warp_smem_bytes = 0;     // dynamic shared memory per warp (replay queue + parking)
+    cudaError_t (*launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
+    // the same with runs that take turns (StepperParams::bench > 0), if there is one
+    const void* bench_func = nullptr;
+    cudaError_t (*bench_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
 };
 
-inline size_t stepper_smem(const StepperKernel& k, int block, int n_sets) {
-    return stepper_table_bytes(n_sets) + (size_t)(block / 32) * (size_t)k.warp_smem_bytes;
+inline size_t stepper_smem(const StepperKernel& k, int block, int n_sets, int bench) {
+    return stepper_table_bytes(n_sets) + (size_t)(block / 32) * (size_t)(k.warp_smem_bytes + bench * kParkWords * 4);
 }
 
 // Block lengths with an instantiation: binary32 8/16/32/64, binary64 4/8; the

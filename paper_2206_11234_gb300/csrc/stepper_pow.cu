@@ -9,17 +9,20 @@ namespace {
 
 constexpr int kPowKS = 32;
 
-template <int PREC, int MODEL, bool WALL>
+template <int PREC, int MODEL, bool WALL, bool BENCH>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
-    const size_t smem = stepper_table_bytes(a.n_sets) + (size_t)(block / 32) * warp_smem_bytes<float, PREC>();
-    stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS><<<grid, block, smem, stream>>>(a);
+    const size_t smem = stepper_table_bytes(a.n_sets) +
+                        (size_t)(block / 32) * (warp_smem_bytes<float, PREC>() + a.bench * kParkWords * 4);
+    stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, BENCH><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
 template <int PREC, int MODEL, bool WALL>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS>,
-                         warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL>};
+    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, false>,
+                         warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, false>,
+                         (const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, true>,
+                         &launch<PREC, MODEL, WALL, true>};
 }
 
 template <int PREC, bool WALL>
@@ -48,10 +51,10 @@ int pow_code(double p) {
 }
 
 StepperKernel stepper_f32_pow(int precision, double p, bool wall, int k_steps) {
-    if (k_steps != kPowKS) return StepperKernel{nullptr, 0, nullptr};
+    if (k_steps != kPowKS) return StepperKernel{};
     if (precision == FPT_PREC_F32_KAHAN) return by_wall<FPT_PREC_F32_KAHAN>(wall, pow_code(p));
     if (precision == FPT_PREC_F32_F64ACC) return by_wall<FPT_PREC_F32_F64ACC>(wall, pow_code(p));
-    return StepperKernel{nullptr, 0, nullptr};
+    return StepperKernel{};
 }
 
 }  // namespace fpt

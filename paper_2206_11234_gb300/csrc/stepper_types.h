@@ -59,6 +59,8 @@ struct SetConst {
     };
 };
 
+constexpr int kParkWords = 12;  // 32-bit words of a run's live state in shared memory
+
 // Bytes of the per-set table at the start of the stepper's dynamic shared
 // memory: n_sets SetConst plus n_sets + 1 set starts, rounded to 16.
 inline __host__ __device__ size_t stepper_table_bytes(int n_sets) {
@@ -83,6 +85,8 @@ struct StepperParams {
     double* out_N;
     double* out_logw;
     StepperScratch* scratch;         // zeroed before the launch
+    int bench;                       // runs that take turns with each warp's 32 (0 .. 32)
+    int bench_every;                 // scheduling blocks between two turns
     unsigned long long* steps_out;   // optional
 };
 

@@ -132,3 +132,34 @@ def test_binary64_caps_inside_a_block(nat, ks, n_max):
     assert np.array_equal(np.isfinite(N), fin)
     assert np.all(np.abs(N[fin] - No[fin]) <= 1e-12 * np.maximum(No[fin], dN))
     assert np.all(np.abs(lw - lwo) <= 1e-12 * np.maximum(1.0, so * b * math.sqrt(dN)))
+
+
+@pytest.mark.parametrize("kind", ["f32_kahan", "f32_f64acc", "power", "quartic"])
+@pytest.mark.parametrize("n", [19457, 20011, 24000, 38913, 40001, 60000])
+def test_runs_that_take_turns(nat, kind, n):
+    """Run counts just above a whole number of warps per scheduler, with runs of one
+    length: the library lets a few runs per warp take turns.  The same records,
+    bit for bit, as in calls small enough that none has to (runs 0 .. n by their
+    offsets), with a second set of runs that start past their end."""
+    import torch
+    kw = {"power": dict(precision="f32_kahan", bias_p=3.0), "quartic": dict(precision="f32_kahan", model=2,
+          poly=[0, 0, 0, 0, 1e-7])}.get(kind, dict(precision=kind))
+    end = 1.8 if kind == "quartic" else W.PHI_END
+    base = dict(m=0.01, dN=5e-4, n_max=0.4 if n == 24000 else 1.0, phi_end=end)  # 24000: censored at the cap
+    specs = [W.SetSpec(phi_in=2.0, b=1e-3, n_traj=n, set_id=4, **base),
+             W.SetSpec(phi_in=1.0, b=1e-3, n_traj=70, set_id=5, **base)]
+    p = nat.make_params(m=0.01, n_max=1.0, **kw)
+
+    def run(sp, seed=6):
+        N = torch.full((sum(s.n_traj for s in sp),), -1.0, dtype=torch.float64, device="cuda")
+        lw = torch.full_like(N, -1.0)
+        nat.fpt_simulate_batch(p, nat.make_sets(sp), seed, N, lw)
+        return N, lw
+
+    N, lw = run(specs)
+    assert torch.all(N[n:] == 0.0) and torch.all(lw[n:] == 0.0)
+    step = 4096
+    for off in range(0, n, step):
+        k = min(step, n - off)
+        N1, l1 = run([W.SetSpec(phi_in=2.0, b=1e-3, n_traj=k, set_id=4, traj_offset=off, **base)])
+        assert torch.equal(N[off:off + k], N1) and torch.equal(lw[off:off + k], l1), off
