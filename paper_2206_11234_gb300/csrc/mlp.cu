@@ -55,52 +55,43 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const fpt_mlp_params* 
     }
 }
 
+// Column sums.  Every parameter gradient but dW2 is a sum over rows of quantities
+// that one thread has for its row.  The rows go to shared memory (h2 in BF16, as the
+// network computes it, delta1 in FP32) and are read back by columns: thread t adds
+// up four columns (4 (t mod 16) ..) of eight rows (8 (t / 16) ..) in registers
+// that live as long as the CTA, and the sixteen row groups meet once, at the end.
+constexpr int kH2Row = 144;  // bytes of a row of h2: 64 bf16 and padding against bank conflicts
+constexpr int kD1Row = 272;  // bytes of a row of delta1: 64 floats and padding
+
 struct MlpBwdSmem {
-    MlpTile f;                                      // A = h1 (rows r, K = k), W2 (rows n, K = k)
-    alignas(128) unsigned char W2T[64 * 64 * 2];    // rows k, K = n
-    alignas(128) unsigned char D2[kTileBytes64];    // delta2: rows r, K = n
-    alignas(128) unsigned char D2T[128 * 128 * 2];  // delta2^T: rows n (64..127 zero), K = r
-    alignas(128) unsigned char H1T[64 * 128 * 2];   // h1^T: rows k, K = r
+    MlpTile f;                                 // A = h1 (rows r, columns k), W2 (rows n, columns k)
+    // delta2 (rows r, columns n) as an operand, then h2; once both have been read,
+    // delta1 takes the place of the two
+    alignas(128) unsigned char D2[kTileBytes64];
+    unsigned char H2[128 * kH2Row];
+    float x[128][2];                           // normalised inputs of the rows
+    float g[128];
     float gw1[kHid][2];
     float gb1[kHid];
     float gb2[kHid];
     float gw3[kHid];
     float gb3;
 };
+static_assert(kTileBytes64 + 128 * kH2Row >= 128 * kD1Row, "delta1 fits over delta2 and h2");
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+constexpr uint32_t kIdescDh1 = tc::idesc_bf16_tn(128, 64, false, true);  // delta2 W2: W2's rows are K
+constexpr uint32_t kIdescDW2 = tc::idesc_bf16_tn(128, 64, true, true);   // delta2^T h1: the tile's rows are K
 
-// Sums of v[0..15] over the 32 lanes of the warp, 16 at once: at each step a
-// lane keeps one half of its values (the upper half when its lane bit is set)
-// and adds its partner's copy of that half, so the values carried halve while
-// the lanes summed double.  Returns in lane L the sum of index L >> 1 (lanes
-// 2u and 2u + 1 both hold index u).  16 shuffles for 16 sums instead of 80.
-// v is overwritten.
-__device__ __forceinline__ float warp_sum16(float v[16]) {
-    const unsigned lane = threadIdx.x & 31u;
-#pragma unroll
-    for (int step = 0; step < 4; ++step) {
-        const int o = 16 >> step, h = 8 >> step;
-        const bool up = (lane & (unsigned)o) != 0u;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const float send = up ? v[i] : v[i + h];
-            const float keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
+// What bounds it: shared-memory accesses (61 % of their rate, ncu) and their
+// latencies around three small products; the tensor pipe idles.  The products read
+// the same tiles in both orders (K-major and MN-major descriptors) instead of
+// transposed copies; that and the column sums replaced 128 two-byte shared accesses
+// and 320 shuffles per row and tile, and 56 KB of copies, so that three CTAs fit
+// where two did.  1,000,003 rows: 280 us with them, 150 us without, 139 us with two
+// threads per row (24 warps per SM instead of 12).
+constexpr int kBwdThreads = 256;  // two threads per row, 32 of the 64 units each
 
-__device__ __forceinline__ void store_bf16(unsigned char* base, uint32_t off, float v) {
-    *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
-}
-
-__global__ void __launch_bounds__(128) mlp_backward_kernel(const fpt_mlp_params* __restrict__ P,
+__global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_mlp_params* __restrict__ P,
                                                            const float* __restrict__ phi,
                                                            const float* __restrict__ N,
                                                            const float* __restrict__ g, long long n,
@@ -116,13 +107,6 @@ __global__ void __launch_bounds__(128) mlp_backward_kernel(const fpt_mlp_params*
         tc::tmem_relinquish();
         tc::fence_before_sync();
     }
-    // W2^T in its tile, zero padding rows of delta2^T, clear the partial sums
-    for (int e = tid; e < 64 * 64; e += blockDim.x) {
-        const int nn = e >> 6, k = e & 63;
-        *reinterpret_cast<uint16_t*>(B.W2T + tc::kmajor_offset(k, nn, 64)) = P->w[kW2 + nn * kHid + k];
-    }
-    for (int e = tid; e < 64 * 128 * 2 / 16; e += blockDim.x)
-        reinterpret_cast<uint4*>(B.D2T + 64 * 128 * 2)[e] = make_uint4(0u, 0u, 0u, 0u);
     for (int j = tid; j < kHid; j += blockDim.x) {
         B.gw1[j][0] = B.gw1[j][1] = 0.f;
         B.gb1[j] = B.gb2[j] = B.gw3[j] = 0.f;
@@ -133,110 +117,132 @@ __global__ void __launch_bounds__(128) mlp_backward_kernel(const fpt_mlp_params*
     uint32_t phase = 0;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
     const long long tiles = (n + 127) / 128;
+    const int row = tid & 127, half = tid >> 7;           // this thread's row and units 32 half ..
+    const int c0 = 4 * (tid & 15), r0 = 8 * (tid >> 4);  // columns and rows of its sums
+    float a_w3[4] = {0.f, 0.f, 0.f, 0.f}, a_b2[4] = {0.f, 0.f, 0.f, 0.f};
+    float a_b1[4] = {0.f, 0.f, 0.f, 0.f}, a_x0[4] = {0.f, 0.f, 0.f, 0.f}, a_x1[4] = {0.f, 0.f, 0.f, 0.f};
+    float a_g = 0.f;
     int done = 0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x, ++done) {
-        const long long i = t * 128 + tid;
+        const long long i = t * 128 + row;
         const bool valid = i < n;
         const float gi = valid ? g[i] : 0.f;
         const float x0 = ((valid ? phi[i] : 0.f) - S.norm[0]) * S.norm[1];
         const float x1 = ((valid ? N[i] : 0.f) - S.norm[2]) * S.norm[3];
-        // layer 1 into A (rows) and H1T (columns)
-        mlp_layer1_to_tile(S, S.A, tid, x0, x1);
-#pragma unroll 8
-        for (int k = 0; k < kHid; ++k) {
-            const uint16_t h = *reinterpret_cast<const uint16_t*>(S.A + tc::kmajor_offset(tid, k, 64));
-            *reinterpret_cast<uint16_t*>(B.H1T + tc::kmajor_offset(k, tid, 128)) = h;
+        if (half == 0) {
+            B.x[row][0] = x0;
+            B.x[row][1] = x1;
+            B.g[row] = gi;
+            a_g += gi;
         }
+        mlp_layer1_to_tile<4>(S, S.A, row, x0, x1, 4 * half);
         tc::fence_proxy_async();
         __syncthreads();
         if (tid == 0) mlp_issue_z2(S);
         if (S.status != 0u || !tc::mbar_wait(&S.mbar, phase)) S.status = 1u;  // one expiry, not one per tile
         phase ^= 1u;
         tc::fence_after_sync();
-        // output layer and delta2
-        for (int c = 0; c < 4; ++c) {
+        // h2 and delta2 = g w3 (1 - h2^2) of the row
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+            const int c = 2 * half + cc;
             float z[16];
             tc::tmem_ld16(S.tmem + lane_base + 16 * c, z);
             tc::tmem_wait_ld();
-            uint32_t q[8];
-            float dd[16], gh[16];
+            uint32_t q[8], hh[8];
 #pragma unroll
             for (int e = 0; e < 16; e += 2) {
                 const int n0 = 16 * c + e;
-                const uint32_t hh = tc::tanh_bf16x2(tc::pack_bf16(z[e] + S.b2[n0], z[e + 1] + S.b2[n0 + 1]));
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int nn = n0 + u;
-                    const float h2 = u == 0 ? tc::bf16_lo(hh) : tc::bf16_hi(hh);
-                    dd[e + u] = gi * S.w3[nn] * (1.f - h2 * h2);
-                    gh[e + u] = gi * h2;
-                    store_bf16(B.D2T, tc::kmajor_offset(nn, tid, 128), dd[e + u]);
-                }
-                q[e / 2] = tc::pack_bf16(dd[e], dd[e + 1]);
+                const uint32_t h = tc::tanh_bf16x2(tc::pack_bf16(z[e] + S.b2[n0], z[e + 1] + S.b2[n0 + 1]));
+                const float h0 = tc::bf16_lo(h), h1 = tc::bf16_hi(h);
+                q[e / 2] = tc::pack_bf16(gi * S.w3[n0] * (1.f - h0 * h0), gi * S.w3[n0 + 1] * (1.f - h1 * h1));
+                hh[e / 2] = h;
             }
-            *reinterpret_cast<uint4*>(B.D2 + tc::kmajor_offset(tid, 16 * c, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4*>(B.D2 + tc::kmajor_offset(tid, 16 * c + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
-            // dw3 += g h2, db2 += delta2, summed over the warp's rows
-            const float sw3 = warp_sum16(gh);
-            const float sb2 = warp_sum16(dd);
-            if ((lane & 1u) == 0u) {
-                atomicAdd(&B.gw3[16 * c + (lane >> 1)], sw3);
-                atomicAdd(&B.gb2[16 * c + (lane >> 1)], sb2);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                *reinterpret_cast<uint4*>(B.D2 + tc::kmajor_offset(row, 16 * c + 8 * u, 64)) =
+                    make_uint4(q[4 * u], q[4 * u + 1], q[4 * u + 2], q[4 * u + 3]);
+                *reinterpret_cast<uint4*>(B.H2 + row * kH2Row + 32 * c + 16 * u) =
+                    make_uint4(hh[4 * u], hh[4 * u + 1], hh[4 * u + 2], hh[4 * u + 3]);
             }
         }
-        const float sg = warp_sum(gi);
-        if (lane == 0) atomicAdd(&B.gb3, sg);
         tc::fence_before_sync();
         tc::fence_proxy_async();
         __syncthreads();
         if (tid == 0) {
             tc::fence_after_sync();
-            const uint32_t d2 = tc::smem_u32(B.D2), w2t = tc::smem_u32(B.W2T);
+            const uint32_t d2 = tc::smem_u32(B.D2), w2 = tc::smem_u32(S.W2), h1 = tc::smem_u32(S.A);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)  // dh1 = delta2 W2 -> columns 0..63
+            for (int kk = 0; kk < 4; ++kk)  // dh1 = delta2 W2 -> columns 0..63, 16 of the n at a time
                 tc::mma_bf16(S.tmem, tc::smem_desc(d2 + 256 * kk, 128, 1024),
-                             tc::smem_desc(w2t + 256 * kk, 128, 1024), kIdescZ2, kk > 0 ? 1u : 0u);
-            const uint32_t d2t = tc::smem_u32(B.D2T), h1t = tc::smem_u32(B.H1T);
+                             tc::smem_desc(w2 + 2048 * kk, 1024, 128), kIdescDh1, kk > 0 ? 1u : 0u);
+            // dW2 += delta2^T h1 -> columns 64..127, 16 rows at a time (of the 128
+            // result rows the first 64 are n; the others hold no result)
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)  // dW2 += delta2^T h1 -> columns 64..127
-                tc::mma_bf16(S.tmem + 64, tc::smem_desc(d2t + 256 * kk, 128, 2048),
-                             tc::smem_desc(h1t + 256 * kk, 128, 2048), kIdescZ2,
-                             (done > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < 8; ++kk)
+                tc::mma_bf16(S.tmem + 64, tc::smem_desc(d2 + 2048 * kk, 1024, 128),
+                             tc::smem_desc(h1 + 2048 * kk, 1024, 128), kIdescDW2, (done > 0 || kk > 0) ? 1u : 0u);
             tc::mma_commit(&S.mbar);
+        }
+        // meanwhile dw3 = sum g h2 and db2 = w3 sum g (1 - h2^2) (w3 at the end)
+#pragma unroll 4
+        for (int r = r0; r < r0 + 8; ++r) {
+            const uint2 h = *reinterpret_cast<const uint2*>(B.H2 + r * kH2Row + 2 * c0);
+            const float gr = B.g[r];
+            const float hv[4] = {tc::bf16_lo(h.x), tc::bf16_hi(h.x), tc::bf16_lo(h.y), tc::bf16_hi(h.y)};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a_w3[u] = fmaf(gr, hv[u], a_w3[u]);
+                a_b2[u] = fmaf(gr, fmaf(-hv[u], hv[u], 1.f), a_b2[u]);
+            }
         }
         if (S.status != 0u || !tc::mbar_wait(&S.mbar, phase)) S.status = 1u;  // one expiry, not one per tile
         phase ^= 1u;
         tc::fence_after_sync();
-        // delta1 and the first-layer gradients
-        for (int c = 0; c < 4; ++c) {
+        __syncthreads();  // h2 has been read: delta1 may take its place
+        // delta1 = dh1 (1 - h1^2) of the row
+        unsigned char* d1 = B.D2;
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+            const int c = 2 * half + cc;
             float dh[16];
             tc::tmem_ld16(S.tmem + lane_base + 16 * c, dh);
             tc::tmem_wait_ld();
-            float d0[16], d1x0[16];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int k = 16 * c + e;
-                const uint16_t hb = *reinterpret_cast<const uint16_t*>(S.A + tc::kmajor_offset(tid, k, 64));
-                const float h1 = __uint_as_float((uint32_t)hb << 16);
-                const float d1 = dh[e] * (1.f - h1 * h1);
-                d0[e] = d1;
-                d1x0[e] = d1 * x0;
-                dh[e] = d1 * x1;  // dh is dead after this element: reuse it for d1 x1
-            }
-            // db1 += delta1, dW1 += delta1 x^T, summed over the warp's rows
-            const float s0 = warp_sum16(d0), s1 = warp_sum16(d1x0), s2 = warp_sum16(dh);
-            if ((lane & 1u) == 0u) {
-                const int k = 16 * c + (int)(lane >> 1);
-                atomicAdd(&B.gb1[k], s0);
-                atomicAdd(&B.gw1[k][0], s1);
-                atomicAdd(&B.gw1[k][1], s2);
+            for (int u = 0; u < 2; ++u) {
+                const uint4 hq = *reinterpret_cast<const uint4*>(S.A + tc::kmajor_offset(row, 16 * c + 8 * u, 64));
+                const uint32_t hw[4] = {hq.x, hq.y, hq.z, hq.w};
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float h0 = tc::bf16_lo(hw[e]), h1 = tc::bf16_hi(hw[e]);
+                    v[2 * e] = dh[8 * u + 2 * e] * (1.f - h0 * h0);
+                    v[2 * e + 1] = dh[8 * u + 2 * e + 1] * (1.f - h1 * h1);
+                }
+                float4* o = reinterpret_cast<float4*>(d1 + row * kD1Row + 64 * c + 32 * u);
+                o[0] = make_float4(v[0], v[1], v[2], v[3]);
+                o[1] = make_float4(v[4], v[5], v[6], v[7]);
             }
         }
         tc::fence_before_sync();
         __syncthreads();
+        // db1 = sum delta1, dW1 = sum delta1 x^T
+#pragma unroll 4
+        for (int r = r0; r < r0 + 8; ++r) {
+            const float4 d = *reinterpret_cast<const float4*>(d1 + r * kD1Row + 4 * c0);
+            const float2 xr = *reinterpret_cast<const float2*>(B.x[r]);
+            const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a_b1[u] += dv[u];
+                a_x0[u] = fmaf(dv[u], xr.x, a_x0[u]);
+                a_x1[u] = fmaf(dv[u], xr.y, a_x1[u]);
+            }
+        }
+        __syncthreads();  // delta1, the inputs and h1 have been read
     }
     tc::fence_after_sync();
-    // dW2 from TMEM rows 0..63 (warps 0 and 1), the vector sums from shared memory
+    // dW2 from TMEM rows 0..63 (warps 0 and 1), the other sums through shared memory
     if (done > 0 && warp < 2) {
         const int nn = 32 * warp + lane;
         for (int c = 0; c < 4; ++c) {
@@ -248,6 +254,16 @@ __global__ void __launch_bounds__(128) mlp_backward_kernel(const fpt_mlp_params*
         }
     }
     if (done > 0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            atomicAdd(&B.gw3[c0 + u], a_w3[u]);
+            atomicAdd(&B.gb2[c0 + u], S.w3[c0 + u] * a_b2[u]);
+            atomicAdd(&B.gb1[c0 + u], a_b1[u]);
+            atomicAdd(&B.gw1[c0 + u][0], a_x0[u]);
+            atomicAdd(&B.gw1[c0 + u][1], a_x1[u]);
+        }
+        atomicAdd(&B.gb3, a_g);
+        __syncthreads();
         for (int j = tid; j < kHid; j += blockDim.x) {
             atomicAdd(&grad[kW1 + 2 * j], B.gw1[j][0]);
             atomicAdd(&grad[kW1 + 2 * j + 1], B.gw1[j][1]);
@@ -269,14 +285,14 @@ __global__ void __launch_bounds__(128) mlp_backward_kernel(const fpt_mlp_params*
 // Grid for a persistent MLP kernel and a check that its resident CTAs cannot
 // ask for more TMEM columns than an SM has (an allocation would then wait for
 // a CTA that never exits).
-int mlp_grid(const void* func, size_t smem, int tmem_cols, long long tiles, int* grid) {
+int mlp_grid(const void* func, int threads, size_t smem, int tmem_cols, long long tiles, int* grid) {
     int n_sm = 0;
     int rc = device_sm_count(&n_sm);
     if (rc) return rc;
     cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "MLP kernel shared memory");
     int per_sm = 0;
-    rc = resident_ctas(func, 128, smem, tmem_cols, &per_sm);
+    rc = resident_ctas(func, threads, smem, tmem_cols, &per_sm);
     if (rc) return rc;
     if (per_sm < 1) return fail(FPT_EUNSUPPORTED, "MLP kernel does not fit on an SM");
     const long long full = (long long)per_sm * n_sm;
@@ -360,7 +376,7 @@ extern "C" int fpt_mlp_forward(const fpt_mlp_params* w, const float* phi, const 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t smem = mlp_fwd_smem_bytes();
     int grid = 0;
-    int rc = mlp_grid((const void*)mlp_forward_kernel, smem, kFwdTmemCols, (n + 127) / 128, &grid);
+    int rc = mlp_grid((const void*)mlp_forward_kernel, 128, smem, kFwdTmemCols, (n + 127) / 128, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
     cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
@@ -383,15 +399,15 @@ extern "C" int fpt_mlp_backward(const fpt_mlp_params* w, const float* phi, const
     if ((reinterpret_cast<uintptr_t>(w) & 15u) != 0) return fail(FPT_EINVAL, "parameters must be 16-byte aligned");
     if (n == 0) return FPT_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t smem = sizeof(MlpBwdSmem) + 1024;
+    const size_t smem = sizeof(MlpBwdSmem);
     int grid = 0;
-    int rc = mlp_grid((const void*)mlp_backward_kernel, smem, kBwdTmemCols, (n + 127) / 128, &grid);
+    int rc = mlp_grid((const void*)mlp_backward_kernel, kBwdThreads, smem, kBwdTmemCols, (n + 127) / 128, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
     cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "MLP status");
     cudaMemsetAsync(d_status, 0, sizeof(unsigned), st);
-    mlp_backward_kernel<<<grid, 128, smem, st>>>(w, phi, N, g, (long long)n, grad, d_status);
+    mlp_backward_kernel<<<grid, kBwdThreads, smem, st>>>(w, phi, N, g, (long long)n, grad, d_status);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         cudaFreeAsync(d_status, st);

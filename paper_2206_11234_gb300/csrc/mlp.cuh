@@ -78,11 +78,14 @@ __device__ __forceinline__ void mlp_tile_load(MlpTile& S, const fpt_mlp_params* 
 }
 
 // First layer of row `row` (this thread) into the A tile: h1 = tanh(W1 x + b1),
-// two units per MUFU operation (bf16x2 tanh; the tile holds bf16 anyway).
+// two units per MUFU operation (bf16x2 tanh; the tile holds bf16 anyway).  Units
+// 8 c0 .. 8 (c0 + C) - 1.
+template <int C = 8>
 __device__ __forceinline__ void mlp_layer1_to_tile(const MlpTile& S, unsigned char* A, int row, float x0,
-                                                   float x1) {
+                                                   float x1, int c0 = 0) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
+    for (int cc = 0; cc < C; ++cc) {
+        const int c = c0 + cc;
         uint32_t q[4];
 #pragma unroll
         for (int p = 0; p < 4; ++p) {

@@ -40,6 +40,15 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same with both operands MN-major: A is read as A^T and B as B^T of tiles stored
+// as above, i.e. D = A^T B with the tiles' rows as the K dimension.  In the no-swizzle
+// MN-major layout a core matrix is 8 K-rows of 16 bytes along M/N, which is the
+// K-major core matrix of the transposed tile; LBO then steps along K (8 rows) and
+// SBO along M/N (8 columns).
+__host__ __device__ constexpr uint32_t idesc_bf16_tn(int M, int N, bool a_mn, bool b_mn) {
+    return idesc_bf16(M, N) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(smem_u32(dst_smem)), "r"(ncols) : "memory");
