@@ -342,7 +342,7 @@ extern "C" int fpt_wait_selftest(int32_t* expired_out, double* seconds_out, void
     if (!expired_out) return fail(FPT_EINVAL, "expired_out is NULL");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     unsigned* d = nullptr;
-    cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&d), sizeof(unsigned), st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d), sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "self-test flag");
     cudaMemsetAsync(d, 0, sizeof(unsigned), st);
     cudaEvent_t a, b;
@@ -379,7 +379,7 @@ extern "C" int fpt_mlp_forward(const fpt_mlp_params* w, const float* phi, const 
     int rc = mlp_grid((const void*)mlp_forward_kernel, 128, smem, kFwdTmemCols, (n + 127) / 128, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
-    cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "MLP status");
     cudaMemsetAsync(d_status, 0, sizeof(unsigned), st);
     mlp_forward_kernel<<<grid, 128, smem, st>>>(w, phi, N, (long long)n, out_b, d_status);
@@ -404,7 +404,7 @@ extern "C" int fpt_mlp_backward(const fpt_mlp_params* w, const float* phi, const
     int rc = mlp_grid((const void*)mlp_backward_kernel, kBwdThreads, smem, kBwdTmemCols, (n + 127) / 128, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
-    cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "MLP status");
     cudaMemsetAsync(d_status, 0, sizeof(unsigned), st);
     mlp_backward_kernel<<<grid, kBwdThreads, smem, st>>>(w, phi, N, g, (long long)n, grad, d_status);

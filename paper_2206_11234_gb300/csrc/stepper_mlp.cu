@@ -384,7 +384,7 @@ extern "C" int fpt_simulate_mlp(const fpt_params* p, const fpt_set* sets, int32_
     workspace_image(P, L, &img);
     const size_t off_cnt = L.bytes;
     unsigned char* ws = nullptr;
-    cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&ws), L.bytes + 256, st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&ws), L.bytes + 256, st);
     if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
     std::vector<unsigned char> img2(img);
     img2.resize(L.bytes + 256, 0);

@@ -170,7 +170,7 @@ extern "C" int fpt_mlp_train_step(const fpt_params* p, const fpt_set* set, uint6
     if (rc) return rc;
     const long long n = set->n_traj;
     TailAcc* acc = nullptr;
-    cudaError_t e = lib_malloc_async(reinterpret_cast<void**>(&acc), sizeof(TailAcc), st);
+    cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&acc), sizeof(TailAcc), st);
     if (e != cudaSuccess) return cuda_fail(e, "training scratch");
     cudaMemsetAsync(acc, 0, sizeof(TailAcc), st);
     int n_sm = 0;
