@@ -79,6 +79,12 @@ struct MlpBwdSmem {
 };
 static_assert(kTileBytes64 + 128 * kH2Row >= 128 * kD1Row, "delta1 fits over delta2 and h2");
 
+// 1 - h^2 of two BF16 values
+__device__ __forceinline__ tc::f32x2 one_minus_square(uint32_t h) {
+    const float lo = tc::bf16_lo(h), hi = tc::bf16_hi(h);
+    return tc::fma2(tc::pair(-lo, -hi), tc::pair(lo, hi), tc::pair(1.f, 1.f));
+}
+
 constexpr uint32_t kIdescDh1 = tc::idesc_bf16_tn(128, 64, false, true);  // delta2 W2: W2's rows are K
 constexpr uint32_t kIdescDW2 = tc::idesc_bf16_tn(128, 64, true, true);   // delta2^T h1: the tile's rows are K
 
@@ -119,8 +125,8 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
     const long long tiles = (n + 127) / 128;
     const int row = tid & 127, half = tid >> 7;           // this thread's row and units 32 half ..
     const int c0 = 4 * (tid & 15), r0 = 8 * (tid >> 4);  // columns and rows of its sums
-    float a_w3[4] = {0.f, 0.f, 0.f, 0.f}, a_b2[4] = {0.f, 0.f, 0.f, 0.f};
-    float a_b1[4] = {0.f, 0.f, 0.f, 0.f}, a_x0[4] = {0.f, 0.f, 0.f, 0.f}, a_x1[4] = {0.f, 0.f, 0.f, 0.f};
+    // two columns each; 0 is two binary32 zeros
+    tc::f32x2 a_w3[2] = {0, 0}, a_b2[2] = {0, 0}, a_b1[2] = {0, 0}, a_x0[2] = {0, 0}, a_x1[2] = {0, 0};
     float a_g = 0.f;
     int done = 0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x, ++done) {
@@ -135,7 +141,7 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
             B.g[row] = gi;
             a_g += gi;
         }
-        mlp_layer1_to_tile<4>(S, S.A, row, x0, x1, 4 * half);
+        mlp_layer1_to_tile<4, 4>(S, S.A, row, x0, x1, 4 * half);
         tc::fence_proxy_async();
         __syncthreads();
         if (tid == 0) mlp_issue_z2(S);
@@ -143,6 +149,7 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
         phase ^= 1u;
         tc::fence_after_sync();
         // h2 and delta2 = g w3 (1 - h2^2) of the row
+        const tc::f32x2 gg = tc::pair(gi, gi);
 #pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
             const int c = 2 * half + cc;
@@ -151,12 +158,18 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
             tc::tmem_wait_ld();
             uint32_t q[8], hh[8];
 #pragma unroll
-            for (int e = 0; e < 16; e += 2) {
+            for (int e = 0; e < 16; e += 4) {
                 const int n0 = 16 * c + e;
-                const uint32_t h = tc::tanh_bf16x2(tc::pack_bf16(z[e] + S.b2[n0], z[e + 1] + S.b2[n0 + 1]));
-                const float h0 = tc::bf16_lo(h), h1 = tc::bf16_hi(h);
-                q[e / 2] = tc::pack_bf16(gi * S.w3[n0] * (1.f - h0 * h0), gi * S.w3[n0 + 1] * (1.f - h1 * h1));
-                hh[e / 2] = h;
+                tc::f32x2 bb[2], w[2];
+                tc::load_pairs(S.b2 + n0, bb[0], bb[1]);
+                tc::load_pairs(S.w3 + n0, w[0], w[1]);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t h = tc::tanh_bf16x2(
+                        tc::pack_bf16(tc::add2(tc::pair(z[e + 2 * k], z[e + 2 * k + 1]), bb[k])));
+                    hh[e / 2 + k] = h;
+                    q[e / 2 + k] = tc::pack_bf16(tc::mul2(tc::mul2(gg, w[k]), one_minus_square(h)));
+                }
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
@@ -188,12 +201,12 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
 #pragma unroll 4
         for (int r = r0; r < r0 + 8; ++r) {
             const uint2 h = *reinterpret_cast<const uint2*>(B.H2 + r * kH2Row + 2 * c0);
-            const float gr = B.g[r];
-            const float hv[4] = {tc::bf16_lo(h.x), tc::bf16_hi(h.x), tc::bf16_lo(h.y), tc::bf16_hi(h.y)};
+            const tc::f32x2 gr = tc::pair(B.g[r], B.g[r]);
+            const uint32_t hw[2] = {h.x, h.y};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a_w3[u] = fmaf(gr, hv[u], a_w3[u]);
-                a_b2[u] = fmaf(gr, fmaf(-hv[u], hv[u], 1.f), a_b2[u]);
+            for (int u = 0; u < 2; ++u) {
+                a_w3[u] = tc::fma2(gr, tc::pair(tc::bf16_lo(hw[u]), tc::bf16_hi(hw[u])), a_w3[u]);
+                a_b2[u] = tc::fma2(gr, one_minus_square(hw[u]), a_b2[u]);
             }
         }
         if (S.status != 0u || !tc::mbar_wait(&S.mbar, phase)) S.status = 1u;  // one expiry, not one per tile
@@ -212,16 +225,14 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
             for (int u = 0; u < 2; ++u) {
                 const uint4 hq = *reinterpret_cast<const uint4*>(S.A + tc::kmajor_offset(row, 16 * c + 8 * u, 64));
                 const uint32_t hw[4] = {hq.x, hq.y, hq.z, hq.w};
-                float v[8];
+                ulonglong2* o = reinterpret_cast<ulonglong2*>(d1 + row * kD1Row + 64 * c + 32 * u);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float h0 = tc::bf16_lo(hw[e]), h1 = tc::bf16_hi(hw[e]);
-                    v[2 * e] = dh[8 * u + 2 * e] * (1.f - h0 * h0);
-                    v[2 * e + 1] = dh[8 * u + 2 * e + 1] * (1.f - h1 * h1);
+                for (int e = 0; e < 2; ++e) {
+                    const int k = 8 * u + 4 * e;
+                    o[e] = make_ulonglong2(
+                        tc::mul2(tc::pair(dh[k], dh[k + 1]), one_minus_square(hw[2 * e])),
+                        tc::mul2(tc::pair(dh[k + 2], dh[k + 3]), one_minus_square(hw[2 * e + 1])));
                 }
-                float4* o = reinterpret_cast<float4*>(d1 + row * kD1Row + 64 * c + 32 * u);
-                o[0] = make_float4(v[0], v[1], v[2], v[3]);
-                o[1] = make_float4(v[4], v[5], v[6], v[7]);
             }
         }
         tc::fence_before_sync();
@@ -229,14 +240,14 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
         // db1 = sum delta1, dW1 = sum delta1 x^T
 #pragma unroll 4
         for (int r = r0; r < r0 + 8; ++r) {
-            const float4 d = *reinterpret_cast<const float4*>(d1 + r * kD1Row + 4 * c0);
+            const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(d1 + r * kD1Row + 4 * c0);
             const float2 xr = *reinterpret_cast<const float2*>(B.x[r]);
-            const float dv[4] = {d.x, d.y, d.z, d.w};
+            const tc::f32x2 dv[2] = {d.x, d.y}, xx0 = tc::pair(xr.x, xr.x), xx1 = tc::pair(xr.y, xr.y);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a_b1[u] += dv[u];
-                a_x0[u] = fmaf(dv[u], xr.x, a_x0[u]);
-                a_x1[u] = fmaf(dv[u], xr.y, a_x1[u]);
+            for (int u = 0; u < 2; ++u) {
+                a_b1[u] = tc::add2(a_b1[u], dv[u]);
+                a_x0[u] = tc::fma2(dv[u], xx0, a_x0[u]);
+                a_x1[u] = tc::fma2(dv[u], xx1, a_x1[u]);
             }
         }
         __syncthreads();  // delta1, the inputs and h1 have been read
@@ -255,12 +266,24 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
     }
     if (done > 0) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            atomicAdd(&B.gw3[c0 + u], a_w3[u]);
-            atomicAdd(&B.gb2[c0 + u], S.w3[c0 + u] * a_b2[u]);
-            atomicAdd(&B.gb1[c0 + u], a_b1[u]);
-            atomicAdd(&B.gw1[c0 + u][0], a_x0[u]);
-            atomicAdd(&B.gw1[c0 + u][1], a_x1[u]);
+        for (int u = 0; u < 2; ++u) {
+            const int k = c0 + 2 * u;
+            float lo, hi;
+            tc::split(a_w3[u], lo, hi);
+            atomicAdd(&B.gw3[k], lo);
+            atomicAdd(&B.gw3[k + 1], hi);
+            tc::split(a_b2[u], lo, hi);
+            atomicAdd(&B.gb2[k], S.w3[k] * lo);
+            atomicAdd(&B.gb2[k + 1], S.w3[k + 1] * hi);
+            tc::split(a_b1[u], lo, hi);
+            atomicAdd(&B.gb1[k], lo);
+            atomicAdd(&B.gb1[k + 1], hi);
+            tc::split(a_x0[u], lo, hi);
+            atomicAdd(&B.gw1[k][0], lo);
+            atomicAdd(&B.gw1[k + 1][0], hi);
+            tc::split(a_x1[u], lo, hi);
+            atomicAdd(&B.gw1[k][1], lo);
+            atomicAdd(&B.gw1[k + 1][1], hi);
         }
         atomicAdd(&B.gb3, a_g);
         __syncthreads();

@@ -35,10 +35,13 @@ constexpr int kTileBytes64 = 128 * 64 * 2;              // 128 rows x K 64, bf16
 struct MlpTile {
     alignas(128) unsigned char A[kTileBytes64];   // h1, rows = threads, K = 64 hidden
     alignas(128) unsigned char W2[64 * 64 * 2];   // rows = output n, K = input k
-    float w1[kHid][2];
-    float b1[kHid];
-    float b2[kHid];
-    float w3[kHid];
+    // by unit, so that four units' values come in one 16-byte read and are worked on
+    // two at a time
+    alignas(16) float w1a[kHid];  // W1[j][0]
+    alignas(16) float w1b[kHid];  // W1[j][1]
+    alignas(16) float b1[kHid];
+    alignas(16) float b2[kHid];
+    alignas(16) float w3[kHid];
     float b3;
     float norm[4];
     uint64_t mbar;
@@ -60,8 +63,8 @@ __device__ __forceinline__ void mlp_tile_load(MlpTile& S, const fpt_mlp_params* 
         *reinterpret_cast<uint4*>(S.W2 + tc::kmajor_offset(n, 8 * c, 64)) = v;
     }
     for (int j = tid; j < kHid; j += blockDim.x) {
-        S.w1[j][0] = bf16_at(P->w, kW1 + 2 * j);
-        S.w1[j][1] = bf16_at(P->w, kW1 + 2 * j + 1);
+        S.w1a[j] = bf16_at(P->w, kW1 + 2 * j);
+        S.w1b[j] = bf16_at(P->w, kW1 + 2 * j + 1);
         S.b1[j] = bf16_at(P->w, kB1 + j);
         S.b2[j] = bf16_at(P->w, kB2 + j);
         S.w3[j] = bf16_at(P->w, kW3 + j);
@@ -79,22 +82,31 @@ __device__ __forceinline__ void mlp_tile_load(MlpTile& S, const fpt_mlp_params* 
 
 // First layer of row `row` (this thread) into the A tile: h1 = tanh(W1 x + b1),
 // two units per MUFU operation (bf16x2 tanh; the tile holds bf16 anyway).  Units
-// 8 c0 .. 8 (c0 + C) - 1.
-template <int C = 8>
+// 8 c0 .. 8 (c0 + C) - 1, BATCH x 8 of them between stores: a store to the tile holds
+// back the reads of the next units' parameters (the compiler cannot tell them apart),
+// so each batch pays its latencies once.
+template <int C = 8, int BATCH = 1>
 __device__ __forceinline__ void mlp_layer1_to_tile(const MlpTile& S, unsigned char* A, int row, float x0,
                                                    float x1, int c0 = 0) {
+    const tc::f32x2 xx0 = tc::pair(x0, x0), xx1 = tc::pair(x1, x1);
 #pragma unroll
-    for (int cc = 0; cc < C; ++cc) {
-        const int c = c0 + cc;
-        uint32_t q[4];
+    for (int cb = 0; cb < C; cb += BATCH) {
+        uint32_t q[4 * BATCH];
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const int j = 8 * c + 2 * p;
-            const float a0 = fmaf(S.w1[j][0], x0, fmaf(S.w1[j][1], x1, S.b1[j]));
-            const float a1 = fmaf(S.w1[j + 1][0], x0, fmaf(S.w1[j + 1][1], x1, S.b1[j + 1]));
-            q[p] = tc::tanh_bf16x2(tc::pack_bf16(a0, a1));
+        for (int p = 0; p < 2 * BATCH; ++p) {
+            const int j = 8 * (c0 + cb) + 4 * p;
+            tc::f32x2 wa[2], wb[2], bb[2];
+            tc::load_pairs(S.w1a + j, wa[0], wa[1]);
+            tc::load_pairs(S.w1b + j, wb[0], wb[1]);
+            tc::load_pairs(S.b1 + j, bb[0], bb[1]);
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                q[2 * p + k] = tc::tanh_bf16x2(tc::pack_bf16(tc::fma2(wa[k], xx0, tc::fma2(wb[k], xx1, bb[k]))));
         }
-        *reinterpret_cast<uint4*>(A + tc::kmajor_offset(row, 8 * c, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
+#pragma unroll
+        for (int c = 0; c < BATCH; ++c)
+            *reinterpret_cast<uint4*>(A + tc::kmajor_offset(row, 8 * (c0 + cb + c), 64)) =
+                make_uint4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
     }
 }
 
@@ -129,11 +141,13 @@ __device__ __forceinline__ void mlp_tile_mma(MlpTile& S, uint32_t& phase, Issue 
 // b(phi, N) for every row of the tile: one call per thread of the 128-thread
 // CTA, all threads together.  `phase` is the mbarrier parity to wait for (all
 // threads keep the same value).  The A tile is free again when this returns.
+// WIDE: all of z2 is read at once, for kernels with registers to spare.
+template <bool WIDE = false>
 __device__ __forceinline__ float mlp_tile_forward(MlpTile& S, float phi, float N, uint32_t& phase) {
     const int tid = threadIdx.x;
     const float x0 = (phi - S.norm[0]) * S.norm[1];
     const float x1 = (N - S.norm[2]) * S.norm[3];
-    mlp_layer1_to_tile(S, S.A, tid, x0, x1);
+    mlp_layer1_to_tile<8, WIDE ? 8 : 1>(S, S.A, tid, x0, x1);
     // z2 = W2 h1 (b2 is added below)
     mlp_tile_mma(S, phase, [&] {
         const uint32_t a = tc::smem_u32(S.A), w2 = tc::smem_u32(S.W2);
@@ -145,17 +159,25 @@ __device__ __forceinline__ float mlp_tile_forward(MlpTile& S, float phi, float N
     // h2 = tanh(z2 + b2) in BF16 (two units per MUFU operation), b = w3 . h2 + b3
     const uint32_t taddr = S.tmem + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16);
     float b = S.b3;
+    constexpr int kCols = WIDE ? 64 : 16;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        float z[16];
-        tc::tmem_ld16(taddr + 16 * c, z);
+    for (int c = 0; c < 64 / kCols; ++c) {
+        float z[kCols];
+#pragma unroll
+        for (int k = 0; k < kCols; k += 16) tc::tmem_ld16(taddr + kCols * c + k, z + k);
         tc::tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-            const int n0 = 16 * c + e;
-            const uint32_t hh = tc::tanh_bf16x2(tc::pack_bf16(z[e] + S.b2[n0], z[e + 1] + S.b2[n0 + 1]));
-            b = fmaf(S.w3[n0], tc::bf16_lo(hh), b);
-            b = fmaf(S.w3[n0 + 1], tc::bf16_hi(hh), b);
+        for (int e = 0; e < kCols; e += 4) {
+            const int n0 = kCols * c + e;
+            tc::f32x2 bb[2];
+            tc::load_pairs(S.b2 + n0, bb[0], bb[1]);
+            const float4 w = *reinterpret_cast<const float4*>(S.w3 + n0);
+            const uint32_t h0 = tc::tanh_bf16x2(tc::pack_bf16(tc::add2(tc::pair(z[e], z[e + 1]), bb[0])));
+            const uint32_t h1 = tc::tanh_bf16x2(tc::pack_bf16(tc::add2(tc::pair(z[e + 2], z[e + 3]), bb[1])));
+            b = fmaf(w.x, tc::bf16_lo(h0), b);
+            b = fmaf(w.y, tc::bf16_hi(h0), b);
+            b = fmaf(w.z, tc::bf16_lo(h1), b);
+            b = fmaf(w.w, tc::bf16_hi(h1), b);
         }
     }
     tc::fence_before_sync();

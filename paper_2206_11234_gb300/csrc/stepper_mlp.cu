@@ -58,10 +58,43 @@ __device__ __forceinline__ void emit_records(const RecordSink& sink, bool want, 
     }
 }
 
-template <int KS>
+// The same through a buffer of kHeld records per thread in shared memory, for
+// launches of few warps: the atomic's round trip of about 900 cycles stalls a warp
+// wherever it is placed (its result shares a scoreboard with the steps' XU
+// operations), so it is made once in kHeld blocks.
+constexpr int kHeld = 16;
+struct HeldRecords {
+    fpt_mlp_record* slot;  // this thread's first, 128 apart
+    int n;                 // held by this thread
+
+    __device__ __forceinline__ void flush(const RecordSink& sink) {
+        const unsigned FULL = 0xffffffffu;
+        const unsigned lane = threadIdx.x & 31u;
+        unsigned long long base = 0;
+        const int total = __reduce_add_sync(FULL, n);
+        if (lane == 0u && total > 0) base = atomicAdd(sink.count, (unsigned long long)total);
+        base = __shfl_sync(FULL, base, 0);
+#pragma unroll
+        for (int k = 0; k < kHeld; ++k) {
+            const unsigned mask = __ballot_sync(FULL, k < n);
+            const unsigned long long at = base + __popc(mask & ((1u << lane) - 1u));
+            if (k < n && at < sink.cap) sink.out[at] = slot[128 * k];
+            base += __popc(mask);
+        }
+        n = 0;
+    }
+    __device__ __forceinline__ void emit(const RecordSink& sink, bool want, float phi0, float N0, float xi,
+                                         unsigned long long rec) {
+        if (!sink.count) return;
+        if (__any_sync(0xffffffffu, n == kHeld)) flush(sink);
+        if (want) slot[128 * n++] = fpt_mlp_record{phi0, N0, xi, (uint32_t)rec};
+    }
+};
+
+template <int KS, bool FEW>
 __device__ __forceinline__ void replay_mlp(const PendingMlp* q, int cnt, const StepperParams& P,
-                                           const SetConst* s_sets, const RecordSink& sink, unsigned lane,
-                                           unsigned long long& my_steps) {
+                                           const SetConst* s_sets, const RecordSink& sink, HeldRecords& held,
+                                           unsigned lane, unsigned long long& my_steps) {
     const unsigned mask = cnt >= 32 ? 0xffffffffu : ((1u << cnt) - 1u);
     bool have = (int)lane < cnt;
     PendingMlp e{};
@@ -109,7 +142,8 @@ __device__ __forceinline__ void replay_mlp(const PendingMlp* q, int cnt, const S
     }
     __syncwarp();
     const float xisum = -kSqrt2Ln2 * s2;  // the block's sum of normals up to the last step
-    emit_records(sink, have, e.phi0, __fmul_rn((float)e.m0, S.f_dN), xisum, e.rec);
+    if constexpr (FEW) held.emit(sink, have, e.phi0, __fmul_rn((float)e.m0, S.f_dN), xisum, e.rec);
+    else emit_records(sink, have, e.phi0, __fmul_rn((float)e.m0, S.f_dN), xisum, e.rec);
     if (!have) return;
     const float bsq = __fmul_rn(e.b, S.f_sq);
     const float hb2 = __fmul_rn(0.5f * e.b, __fmul_rn(e.b, S.f_dN));
@@ -126,14 +160,20 @@ __device__ __forceinline__ void replay_mlp(const PendingMlp* q, int cnt, const S
     my_steps += (unsigned long long)M;
 }
 
-// The bound caps the kernel at 64 registers (16 bytes spilled; 72 without
-// it), for a schedule that waits less on dependencies (6.93e11 against
-// 6.80e11 steps/s on the learned-bias workload when measured).  Residency is
-// 6 CTAs per SM, set by the ~34.5 KB of shared memory each holds (the tile's
-// 26 KB of operands and parameters and 8 KB of replay queues); at 5 CTAs,
-// with the earlier three-MMA tile of 44 KB, the kernel ran at the same speed.
-template <int KS>
-__global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams P, const fpt_mlp_params* __restrict__ W,
+// Many runs: the bound caps the kernel at 64 registers (a few bytes spilled; 72
+// without it), for a schedule that waits less on dependencies (6.93e11 against
+// 6.80e11 steps/s on the learned-bias workload when measured).  Residency is 6 CTAs
+// per SM, set by the ~34.5 KB of shared memory each holds (the tile's 26 KB of
+// operands and parameters and 8 KB of replay queues).
+//
+// FEW: at most two CTAs per SM (a training batch of 2^14 runs is 128 CTAs), where
+// nothing hides a latency: a block of 32 steps then took 6300 cycles, 2114 in its
+// steps (the chain of a run), 1292 and 1148 in the two layers around the 513 of the
+// product, 1175 in the records' atomic.  With registers to spare the layers load and
+// issue ahead (828 and 780; each has 512 cycles of XU work), and records are held
+// back (HeldRecords): 4700 cycles.
+template <int KS, bool FEW>
+__global__ void __launch_bounds__(128, FEW ? 2 : 8) stepper_mlp_kernel(const StepperParams P, const fpt_mlp_params* __restrict__ W,
                                                           const RecordSink sink) {
     extern __shared__ __align__(1024) unsigned char s_dyn[];
     MlpTile& F = *reinterpret_cast<MlpTile*>(s_dyn);
@@ -144,6 +184,7 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
     unsigned char* s_queue = s_dyn + off_sets + stepper_table_bytes(n_sets);
     const unsigned tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u, lt_mask = (1u << lane) - 1u;
     PendingMlp* q = reinterpret_cast<PendingMlp*>(s_queue) + warp * kQueueCap;
+    HeldRecords held{reinterpret_cast<fpt_mlp_record*>(s_queue + 4 * kQueueCap * sizeof(PendingMlp)) + tid, 0};
     // lane state parked during a replay lives in the MLP's A tile, which holds
     // nothing between two bias evaluations (mlp_tile_forward waits for the
     // last MMA that reads it)
@@ -222,7 +263,7 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
 
         // ---- the learned bias at the block start, 128 runs per tensor-core tile ----
         const SetConst& S = s_sets[set];
-        const float b = mlp_tile_forward(F, phi, __fmul_rn((float)m, S.f_dN), phase);
+        const float b = mlp_tile_forward<FEW>(F, phi, __fmul_rn((float)m, S.f_dN), phase);
         model.tc = __fmul_rn(b, S.f_cmdN);
 
         // ---- one block of KS steps ----
@@ -243,7 +284,8 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
             const float hb2 = __fmul_rn(0.5f * b, __fmul_rn(b, S.f_dN));
             lw += (double)(-bsq * sblk - hb2 * (float)KS);
         }
-        emit_records(sink, through, phi0, __fmul_rn((float)m0, S.f_dN), sblk, rec);
+        if constexpr (FEW) held.emit(sink, through, phi0, __fmul_rn((float)m0, S.f_dN), sblk, rec);
+        else emit_records(sink, through, phi0, __fmul_rn((float)m0, S.f_dN), sblk, rec);
         const unsigned ev = __ballot_sync(FULL, event);
         if (ev) {
             if (event) {
@@ -269,7 +311,7 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
                 park(v, 8 * stride, pl.r1_x1);
                 park(v, 9 * stride, pl.r1_set);
                 __syncwarp();
-                replay_mlp<KS>(q, 32, P, s_sets, sink, lane, my_steps);
+                replay_mlp<KS, FEW>(q, 32, P, s_sets, sink, held, lane, my_steps);
                 __syncwarp();
                 const int rest = q_count - 32;
                 PendingMlp tmp;
@@ -299,7 +341,13 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
     }
     if (q_count > 0) {
         __syncwarp();
-        replay_mlp<KS>(q, q_count, P, s_sets, sink, lane, my_steps);
+        replay_mlp<KS, FEW>(q, q_count, P, s_sets, sink, held, lane, my_steps);
+    }
+    if constexpr (FEW) {
+        if (sink.count) {
+            __syncwarp();
+            held.flush(sink);
+        }
     }
     __syncwarp();
 #pragma unroll
@@ -318,32 +366,35 @@ __global__ void __launch_bounds__(128, 8) stepper_mlp_kernel(const StepperParams
     }
 }
 
-size_t stepper_mlp_smem(int n_sets) {
-    return (sizeof(MlpTile) + 15) / 16 * 16 + stepper_table_bytes(n_sets) + 4 * kQueueCap * sizeof(PendingMlp);
-}
-
-template <int KS>
-int launch_mlp(const StepperParams& a, const fpt_mlp_params* W, const RecordSink& sink, int n_sets,
-               cudaStream_t st) {
-    const void* func = (const void*)stepper_mlp_kernel<KS>;
-    const size_t smem = stepper_mlp_smem(n_sets);
-    int n_sm = 0;
-    int rc = device_sm_count(&n_sm);
-    if (rc) return rc;
+template <int KS, bool FEW>
+int launch_variant(const StepperParams& a, const fpt_mlp_params* W, const RecordSink& sink, int n_sm,
+                   cudaStream_t st) {
+    const void* func = (const void*)stepper_mlp_kernel<KS, FEW>;
+    const size_t smem = (sizeof(MlpTile) + 15) / 16 * 16 + stepper_table_bytes(a.n_sets) +
+                        4 * kQueueCap * sizeof(PendingMlp) + (FEW ? 128 * kHeld * sizeof(fpt_mlp_record) : 0);
     cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "learned-bias stepper shared memory");
     // every resident CTA holds kMlpTmemCols TMEM columns until it exits
     int per_sm = 0;
-    rc = resident_ctas(func, 128, smem, kMlpTmemCols, &per_sm);
+    int rc = resident_ctas(func, 128, smem, kMlpTmemCols, &per_sm);
     if (rc) return rc;
     if (per_sm < 1) return fail(FPT_EUNSUPPORTED, "learned-bias stepper does not fit on an SM");
     const unsigned long long full = (unsigned long long)per_sm * n_sm;
     const unsigned long long need = (a.n_total + 127) / 128;
     const int grid = (int)(need < full ? (need < 1 ? 1 : need) : full);
-    stepper_mlp_kernel<KS><<<grid, 128, smem, st>>>(a, W, sink);
+    stepper_mlp_kernel<KS, FEW><<<grid, 128, smem, st>>>(a, W, sink);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "learned-bias stepper launch");
     return FPT_OK;
+}
+
+template <int KS>
+int launch_mlp(const StepperParams& a, const fpt_mlp_params* W, const RecordSink& sink, cudaStream_t st) {
+    int n_sm = 0;
+    const int rc = device_sm_count(&n_sm);
+    if (rc) return rc;
+    if (a.n_total <= 2ull * 128ull * (unsigned long long)n_sm) return launch_variant<KS, true>(a, W, sink, n_sm, st);
+    return launch_variant<KS, false>(a, W, sink, n_sm, st);
 }
 
 }  // namespace
@@ -406,10 +457,10 @@ extern "C" int fpt_simulate_mlp(const fpt_params* p, const fpt_set* sets, int32_
     sink.count = records ? reinterpret_cast<unsigned long long*>(ws + off_cnt) : nullptr;
     const fpt_mlp_params* W = static_cast<const fpt_mlp_params*>(p->mlp);
     if (!rc) {
-        if (ks == 16) rc = launch_mlp<16>(a, W, sink, a.n_sets, st);
-        else if (ks == 32) rc = launch_mlp<32>(a, W, sink, a.n_sets, st);
-        else if (ks == 64) rc = launch_mlp<64>(a, W, sink, a.n_sets, st);
-        else rc = launch_mlp<128>(a, W, sink, a.n_sets, st);
+        if (ks == 16) rc = launch_mlp<16>(a, W, sink, st);
+        else if (ks == 32) rc = launch_mlp<32>(a, W, sink, st);
+        else if (ks == 64) rc = launch_mlp<64>(a, W, sink, st);
+        else rc = launch_mlp<128>(a, W, sink, st);
     }
     StepperScratch host;
     unsigned long long count = 0;

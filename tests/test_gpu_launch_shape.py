@@ -163,3 +163,31 @@ def test_runs_that_take_turns(nat, kind, n):
         k = min(step, n - off)
         N1, l1 = run([W.SetSpec(phi_in=2.0, b=1e-3, n_traj=k, set_id=4, traj_offset=off, **base)])
         assert torch.equal(N[off:off + k], N1) and torch.equal(lw[off:off + k], l1), off
+
+
+@pytest.mark.parametrize("k_eval", [16, 32, 64, 128])
+def test_learned_bias_few_and_many_runs(nat, k_eval):
+    """A learned-bias call of few runs takes the kernel with held-back records, one
+    of many runs (more than two tiles of 128 per SM) the other: the same runs and the
+    same set of training records, bit for bit, split at an odd place."""
+    import torch
+    n, cut = 45001, 20011
+    w = nat.mlp_pack(W.mlp_params(seed=21, gain=1.0, out_scale=0.6), (3.0, 1.0, 2.0, 0.5))
+    base = dict(phi_in=2.4, m=1.0, b=0.0, dN=2e-3, n_max=1.0, phi_uv=2.6, set_id=2)
+    p = nat.make_params(precision="f32_f64acc", m=1.0, n_max=1.0, mlp=w, k_eval=k_eval)
+
+    def run(off, k):
+        N = torch.empty(k, dtype=torch.float64, device="cuda")
+        lw = torch.empty_like(N)
+        rec = torch.empty((k * (500 // k_eval + 2), 4), dtype=torch.float32, device="cuda")
+        m = nat.fpt_simulate_mlp(p, nat.make_sets([W.SetSpec(n_traj=k, traj_offset=off, **base)]), 8, N, lw, rec)
+        r = rec[:m].cpu().numpy().view(np.uint32).copy()
+        r[:, 3] += off  # runs are numbered within a call
+        return N, lw, r
+
+    N, lw, r = run(0, n)
+    a, b = run(0, cut), run(cut, n - cut)
+    assert torch.equal(N, torch.cat([a[0], b[0]])) and torch.equal(lw, torch.cat([a[1], b[1]]))
+    both = np.concatenate([a[2], b[2]])
+    order = lambda q: q[np.lexsort(q.T)]  # noqa: E731
+    assert r.shape == both.shape and np.array_equal(order(r), order(both))
