@@ -485,6 +485,7 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
     int n_sm = 0;
     int rc = device_sm_count(&n_sm);
     if (rc) return rc;
+    shape->n_sm = n_sm;
     const double share = len.total / (32.0 * n_sm);
     const int fixed = shape->block;
     // many runs: 256 threads (up to 1 % faster); fewer: 128 (3 x 45,000 equal runs 1652 us, 1774 with
@@ -514,6 +515,13 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
             shape->grid = (int)std::min(need, room);
         }
         if (fixed) break;
+    }
+    // up to three chain warps per SM (stepper_few.cuh, with the measurements)
+    if (k.few_func && !fixed && n_total <= 3ull * 32ull * (unsigned long long)n_sm) {
+        shape->few = true;
+        shape->block = kFewThreads;
+        shape->grid = (int)std::max(1ull, (n_total + 31) / 32);
+        return FPT_OK;
     }
     if (!k.bench_func || uneven || !(len.tail <= 0.1 * len.longest)) return FPT_OK;
     const int b = fixed ? fixed : 128, warps = b / 32;
@@ -607,9 +615,10 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
     a.scratch = reinterpret_cast<StepperScratch*>(ws + L.off_scratch);
     a.bench = shape.bench;
     a.bench_every = shape.bench_every;
+    a.n_sm = shape.n_sm;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
     if (P.n_total > 0) {
-        cudaError_t e = (shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
+        cudaError_t e = (shape.few ? k.few_launch : shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
         if (e != cudaSuccess) return cuda_fail(e, "stepper launch");
     }
     if (after_stepper) {

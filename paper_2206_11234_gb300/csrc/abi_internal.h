@@ -50,7 +50,7 @@ struct RunLengths {
 };
 constexpr long long kTrailingRuns = 1 << 17;  // about the lanes of one GPU
 
-constexpr int kMaxDynSmem = 227 * 1024;  // opt-in limit per block
+constexpr int kMaxDynSmem = 226 * 1024;  // opt-in limit per block, less a kernel's few bytes of static shared memory
 
 // Host-side image of one batched call.
 struct Prepared {
@@ -87,6 +87,8 @@ struct LaunchShape {
     int block = 0, grid = 0;  // block: 0 where stepper_grid may choose it
     int bench = 0;            // runs that take turns with each warp's 32 ...
     int bench_every = 0;      // ... every so many scheduling blocks
+    bool few = false;         // the stepper for few runs
+    int n_sm = 1;
 };
 int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsigned long long n_total,
                  const RunLengths& len, LaunchShape* shape);

@@ -174,11 +174,13 @@ struct ModelStep<float, MODEL> {
         else if constexpr (p == 4) return __fmul_rn(__fmul_rn(phi, phi), phi);
         else return ex2_approx(__fmul_rn(pm1, lg2_approx(phi)));
     }
-    // one step from phi with noise factor q trig; adds the step's log-weight to acc
+    // one step from phi with noise factor g = q trig; adds the step's log-weight to acc
     __device__ __forceinline__ float advance(float phi, float q, float trig, float& acc) const {
+        return advance_g(phi, __fmul_rn(q, trig), acc);
+    }
+    __device__ __forceinline__ float advance_g(float phi, float g, float& acc) const {
         const float inv = rcp_approx(phi);
         const float u = u_of(phi, inv);
-        const float g = __fmul_rn(q, trig);
         const float t = __fmaf_rn(tc, u, g);
         acc = __fmaf_rn(u, __fmaf_rn(a2, u, __fmul_rn(a1, g)), acc);
         return __fadd_rn(phi, __fmaf_rn(phi, t, __fmul_rn(m2dN, inv)));

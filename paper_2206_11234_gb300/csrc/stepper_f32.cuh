@@ -2,6 +2,7 @@
 // log-weight sums per translation unit.
 #pragma once
 #include "stepper.cuh"
+#include "stepper_few.cuh"
 #include "stepper_launch.h"
 
 namespace fpt {
@@ -18,12 +19,20 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 }
 
 template <int PREC, int MODEL, bool WALL, int FOLD>
+cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
+    stepper_few_kernel<PREC, MODEL, WALL, FOLD><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <int PREC, int MODEL, bool WALL, int FOLD>
 StepperKernel make() {
     StepperKernel k{(const void*)stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD, false>,
                     warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, FOLD, false>};
     if constexpr (MODEL == FPT_MODEL_QUADRATIC || MODEL == kModelPolyLow) {
         k.bench_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD, true>;
         k.bench_launch = &launch<PREC, MODEL, WALL, FOLD, true>;
+        k.few_func = (const void*)stepper_few_kernel<PREC, MODEL, WALL, FOLD>;
+        k.few_launch = &launch_few<PREC, MODEL, WALL, FOLD>;
     }
     return k;
 }

@@ -1,0 +1,217 @@
+// Binary32 stepper for few runs: one warp of a CTA steps 32 runs, three compute
+// their noise.
+//
+// A warp that has its scheduler to itself is not bound by a pipe but by its own
+// order: in the persistent stepper (stepper.cuh) it takes 55 to 65 cycles per step,
+// of which the run's chain, reciprocal, multiply-add and add, is 28; the noise's
+// XU operations queue in front of the chain's reciprocal and share its
+// scoreboards.  Here the chain is alone in its warp: the noise warps, on the SM's
+// other schedulers, write what a step needs of each Box–Muller pair to shared
+// memory, every third 16-step group each, and the chain warp reads it one group
+// ahead: 28 cycles per step and some 90 per group for the hand-over.  The numbers,
+// their order and so the records are those of the persistent stepper, bit for bit.
+// us, persistent -> this, at one and at three chain warps per SM (4864, 14,592 runs):
+// power 2423 -> 1783, 2409 -> 2206; wall 3891 -> 2903, 3862 -> 3455; ladder
+// 293 -> 232, 279 -> 263; quartic 151 -> 110, 137 -> 119; diffusive 1057 -> 917 at
+// three; 512 runs to N = 1 156 -> 116.  With four per SM the noise warps contend with the
+// chains (0.93 to 1.19 times as fast), with six they lose (0.71 to 1.0).
+// Slots of two groups read without the copy ahead measured 3 to 9 % slower.
+//
+// Runs are handed out once, 32 to a CTA; all of a warp are at the same step, which
+// is what lets the noise run ahead of them.
+#pragma once
+#include "stepper.cuh"
+
+namespace fpt {
+
+constexpr int kNoiseWarps = 3;
+static_assert(kFewThreads == 32 * (1 + kNoiseWarps), "one chain warp and its noise warps");
+constexpr size_t kRingBytes = (size_t)kNoiseWarps * 8 * 32 * sizeof(float4);  // [slot][pair][lane]
+
+// Hand-over of a slot between its noise warp and the chain warp, 64 threads each:
+// one side arrives and goes on, the other waits for it.
+__device__ __forceinline__ void hand_arrive(int id) {
+    __syncwarp();
+    asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void hand_wait(int id) {
+    __syncwarp();
+    asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ int full_id(int slot) { return 1 + slot; }
+__device__ __forceinline__ int empty_id(int slot) { return 1 + kNoiseWarps + slot; }
+
+template <typename Real, int PREC>
+constexpr size_t few_smem_bytes(int n_sets) {
+    return stepper_table_bytes(n_sets) + kRingBytes + 32 * sizeof(Pending<Real, PREC>);
+}
+
+template <int PREC, int MODEL, bool WALL, int FOLD>
+__global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperParams P) {
+    using Entry = Pending<float, PREC>;
+    static_assert(FOLD % 16 == 0, "a fold is a whole number of 16-step groups");
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ volatile int s_stop[kNoiseWarps];
+    const int n_sets = P.n_sets;
+    SetConst* s_sets = reinterpret_cast<SetConst*>(s_dyn);
+    long long* s_first = reinterpret_cast<long long*>(s_dyn + (size_t)n_sets * sizeof(SetConst));
+    float4* ring = reinterpret_cast<float4*>(s_dyn + stepper_table_bytes(n_sets));
+    Entry* q = reinterpret_cast<Entry*>(s_dyn + stepper_table_bytes(n_sets) + kRingBytes);
+    for (int i = threadIdx.x; i < n_sets; i += blockDim.x) {
+        s_sets[i] = P.sets[i];
+        s_first[i] = P.sets[i].ticket0;
+    }
+    if (threadIdx.x < kNoiseWarps) s_stop[threadIdx.x] = 0;
+    __syncthreads();
+
+    const unsigned FULL = 0xffffffffu;
+    const unsigned lane = threadIdx.x & 31u;
+    const int warp = (int)(threadIdx.x >> 5);
+    // the chain warps of the CTAs that share an SM (b, b + n_sm, ...) on different schedulers
+    const int chain = (int)((blockIdx.x / (unsigned)P.n_sm) % (1 + kNoiseWarps));
+
+    // this lane's run: ticket 32 blockIdx + lane, the last set s with ticket0[s] <= ticket
+    const unsigned long long t = 32ull * blockIdx.x + lane;
+    const bool have = t < P.n_total;
+    int lo = 0, hi = n_sets - 1;
+    while (have && lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((long long)t >= s_first[mid]) lo = mid; else hi = mid - 1;
+    }
+    const SetConst& S = s_sets[lo];
+    const unsigned long long i = have ? t - (unsigned long long)s_first[lo] : 0ull;
+    typename StepOf<float, MODEL>::type model;
+    model.load(S);
+
+    if (warp != chain) {
+        // ---- a noise warp: groups slot, slot + 3, ... until told to stop ----
+        const int slot = (warp - chain + kNoiseWarps) % (1 + kNoiseWarps);
+        const PhiloxLane pl = philox_lane(S.traj_offset + i, S.set_id, P.keys);
+        float4* out = ring + slot * 8 * 32 + lane;
+        for (uint32_t G = (uint32_t)slot;; G += kNoiseWarps) {
+            uint32_t V[12];
+            philox_group(pl, G, P.keys, V);
+            float4 f[8];
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const NormalPair np = group_pair_f32(V, p >> 1, p & 1);
+                const float q2 = __fmul_rn(model.kq, np.rho);
+                if constexpr (is_pow_model(MODEL))
+                    f[p] = make_float4(__fmul_rn(q2, np.c), __fmul_rn(q2, np.s), 0.f, 0.f);
+                else
+                    f[p] = make_float4(__fmaf_rn(q2, np.c, model.tc), __fmaf_rn(q2, np.s, model.tc), np.rho,
+                                       np.c + np.s);
+            }
+            if (G >= (uint32_t)kNoiseWarps) {
+                hand_wait(empty_id(slot));
+                if (s_stop[slot] != 0) return;
+            }
+#pragma unroll
+            for (int p = 0; p < 8; ++p) out[32 * p] = f[p];
+            hand_arrive(full_id(slot));
+        }
+    }
+
+    // ---- the chain warp ----
+    bool on = have;
+    if (have && S.phi_in <= S.phi_end) {
+        // starts at or below the end of inflation: N = 0, w = 1
+        P.out_N[S.first + (long long)i] = 0.0;
+        P.out_logw[S.first + (long long)i] = 0.0;
+        on = false;
+    }
+    const bool ran = on;
+    float phi = set_phi_in<float, MODEL>(S);
+    const float phi_end = set_phi_end<float, MODEL>(S), twouv = set_twouv<float, MODEL>(S);
+    const int m_max = S.m_max;
+    // the state at the last fold before the run's end, as the persistent stepper leaves it
+    float phi0 = phi, mn = phi, acc = 0.f;
+    int m0 = 0;
+    WSum<PREC> W;
+    W.reset();
+    unsigned long long my_steps = 0;
+
+    int slot = 0;  // of the next group to take
+    auto take = [&](float4 f[8]) {
+        hand_wait(full_id(slot));
+#pragma unroll
+        for (int p = 0; p < 8; ++p) f[p] = ring[(slot * 8 + p) * 32 + (int)lane];
+    };
+    auto release = [&]() {
+        hand_arrive(empty_id(slot));
+        slot = slot + 1 == kNoiseWarps ? 0 : slot + 1;
+    };
+    int m = 0;  // steps done
+    // 16 steps; false once every run has finished
+    auto group = [&](const float4 f[8]) -> bool {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            float first;
+            if constexpr (is_pow_model(MODEL)) {
+                phi = model.advance_g(phi, f[p].x, acc);
+                if constexpr (WALL) phi = fminf(phi, twouv - phi);
+                first = phi;
+                phi = model.advance_g(phi, f[p].y, acc);
+                if constexpr (WALL) phi = fminf(phi, twouv - phi);
+            } else {
+                phi = step1_f32<WALL>(model, phi, f[p].x, twouv);
+                first = phi;
+                phi = step1_f32<WALL>(model, phi, f[p].y, twouv);
+                acc = __fmaf_rn(f[p].z, f[p].w, acc);
+            }
+            mn = min3f(mn, first, phi);
+        }
+        m += 16;
+        if (m % FOLD != 0) return true;
+        on = on && !(mn <= phi_end) && m < m_max;
+        WSum<PREC> Wn = W;
+        Wn.add(acc);
+        W.take(Wn, on);
+        acc = 0.f;
+        phi0 = on ? phi : phi0;
+        m0 = on ? m : m0;
+        return __any_sync(FULL, on);
+    };
+    if (__any_sync(FULL, on)) {
+        float4 a[8], b[8];
+        take(a);
+        release();
+        for (;;) {
+            take(b);  // one group ahead: the reads return during the steps
+            if (!group(a)) break;
+            release();
+            take(a);
+            if (!group(b)) break;
+            release();
+        }
+        release();
+    }
+    // the three groups that the noise warps have ready, or will have, are not wanted any more
+#pragma unroll
+    for (int k = 0; k < kNoiseWarps; ++k) {
+        hand_wait(full_id(slot));
+        s_stop[slot] = 1;
+        __syncwarp();
+        release();
+    }
+    const unsigned runs = __ballot_sync(FULL, ran);
+    if (ran) {
+        Entry& e = q[__popc(runs & ((1u << lane) - 1u))];
+        e.rec = (unsigned long long)S.first + i;
+        e.m0 = m0;
+        e.set = lo;
+        e.phi0 = phi0;
+        e.W = W;
+    }
+    __syncwarp();
+    replay_batch<float, PREC, MODEL, WALL, FOLD>(q, __popc(runs), P, s_sets, lane, my_steps);
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) my_steps += __shfl_xor_sync(FULL, my_steps, o);
+    if (lane == 0) {
+        atomicAdd(&P.scratch->steps, my_steps);
+        if (P.steps_out) atomicAdd(P.steps_out, my_steps);
+    }
+}
+
+}  // namespace fpt

@@ -450,6 +450,7 @@ extern "C" int fpt_simulate_mlp(const fpt_params* p, const fpt_set* sets, int32_
     a.out_logw = out_logw;
     a.scratch = reinterpret_cast<StepperScratch*>(ws + L.off_scratch);
     a.bench = a.bench_every = 0;
+    a.n_sm = 1;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
     RecordSink sink;
     sink.out = records;

@@ -2,6 +2,7 @@
 // bias B = A_p phi^p (§3.4 Eq. (26)): p in 0..4 specialised, any other real p
 // through exp2/log2; one scheduling block length (32 steps).
 #include "stepper.cuh"
+#include "stepper_few.cuh"
 #include "stepper_launch.h"
 
 namespace fpt {
@@ -18,11 +19,19 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 }
 
 template <int PREC, int MODEL, bool WALL>
+cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
+    stepper_few_kernel<PREC, MODEL, WALL, kPowKS><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <int PREC, int MODEL, bool WALL>
 StepperKernel make() {
     return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, false>,
                          warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, false>,
                          (const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, true>,
-                         &launch<PREC, MODEL, WALL, true>};
+                         &launch<PREC, MODEL, WALL, true>,
+                         (const void*)stepper_few_kernel<PREC, MODEL, WALL, kPowKS>,
+                         &launch_few<PREC, MODEL, WALL>};
 }
 
 template <int PREC, bool WALL>

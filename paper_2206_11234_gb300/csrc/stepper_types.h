@@ -9,6 +9,7 @@
 namespace fpt {
 
 constexpr int kStepperMaxThreads = 512;
+constexpr int kFewThreads = 128;  // of the stepper for few runs
 
 // Model tags of the quadratic potential with the power-law bias B = A_p phi^p
 // (§3.4 Eq. (26)): kModelPow + p for an integer p in 0..4 (phi^(p-1) by
@@ -87,6 +88,7 @@ struct StepperParams {
     StepperScratch* scratch;         // zeroed before the launch
     int bench;                       // runs that take turns with each warp's 32 (0 .. 32)
     int bench_every;                 // scheduling blocks between two turns
+    int n_sm;                        // SMs of the device
     unsigned long long* steps_out;   // optional
 };
 

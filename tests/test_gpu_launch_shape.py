@@ -191,3 +191,35 @@ def test_learned_bias_few_and_many_runs(nat, k_eval):
     both = np.concatenate([a[2], b[2]])
     order = lambda q: q[np.lexsort(q.T)]  # noqa: E731
     assert r.shape == both.shape and np.array_equal(order(r), order(both))
+
+
+@pytest.mark.parametrize("kind", ["f32_kahan", "f32_f64acc", "power", "power_real", "quartic"])
+@pytest.mark.parametrize("n", [1, 31, 33, 4097])
+@pytest.mark.parametrize("k_steps", [16, 32, 64])
+def test_few_runs(nat, kind, n, k_steps):
+    """Few runs take the stepper with separate noise warps; a caller's block_dim
+    keeps the persistent one.  The same records, bit for bit: sets with and without
+    a wall, at the cap, ended at their start, and an empty one, with caps at and off
+    the edges of 16 and k_steps."""
+    import torch
+    kw = {"power": dict(precision="f32_kahan", bias_p=3.0), "power_real": dict(precision="f32_f64acc", bias_p=2.5),
+          "quartic": dict(precision="f32_kahan", model=2, poly=[0, 0, 0, 0, 0.01])}.get(kind, dict(precision=kind))
+    ks = 32 if kind.startswith("power") else k_steps
+    base = dict(m=1.0, dN=2e-3, phi_end=1.8)
+    specs = [W.SetSpec(phi_in=2.0, b=0.02, n_traj=n, set_id=1, n_max=3.0, **base),
+             W.SetSpec(phi_in=1.9, b=0.01, n_traj=n, set_id=2, n_max=0.13, phi_uv=1.95, **base),
+             W.SetSpec(phi_in=1.7, b=0.01, n_traj=5, set_id=3, n_max=0.13, **base),
+             W.SetSpec(phi_in=1.9, b=0.0, n_traj=0, set_id=4, n_max=0.13, **base),
+             W.SetSpec(phi_in=4.0, b=0.0, n_traj=n, set_id=5, n_max=0.128, **base)]
+    total = 3 * n + 5
+    out = []
+    for block in (0, 128):
+        N = torch.full((total,), -1.0, dtype=torch.float64, device="cuda")
+        lw = torch.full_like(N, -1.0)
+        steps = torch.zeros(1, dtype=torch.int64, device="cuda")
+        p = nat.make_params(m=1.0, n_max=3.0, block_dim=block, k_steps=ks, steps_out=steps, **kw)
+        nat.fpt_simulate_batch(p, nat.make_sets(specs), 12, N, lw)
+        out.append((N, lw, int(steps.item())))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert out[0][2] == out[1][2]
+    assert torch.all(out[0][0][2 * n:2 * n + 5] == 0.0) and torch.all(torch.isinf(out[0][0][2 * n + 5:]))
