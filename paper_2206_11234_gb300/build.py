@@ -111,8 +111,8 @@ def f64_tables() -> str:
 
 
 def exp_table() -> str:
-    """The exponential's table of csrc/histogram.cu: 2^(j/4096), rounded correctly,
-    and ln 2 / 4096 as a 30-bit head and a binary64 tail."""
+    """The exponential's table of csrc/histogram.cu: 2^(-j/4096) in units of 2^-62, ln 2 / 4096
+    in units of 2^-98 as three words, and 4096 / ln 2 in units of 2^-19."""
     bits = 200
     one = 1 << bits
     root = 2 * one
@@ -124,14 +124,14 @@ def exp_table() -> str:
         t //= 9
         k += 2
     step = ln2 >> 12
-    head = step >> (bits - 42) << (bits - 42)  # step ~ 2^-12.5: 30 bits
     x, table = one, []
     for _ in range(1 << 12):
-        table.append((x / one).hex())
-        x = x * root >> bits
-    return ("__device__ const double kExp64[4096] = {%s};\nconstexpr double kExpStepHi = %s, kExpStepLo = %s, "
-            "kExpPerStep = %s;\n" % (",".join(table), (head / one).hex(), ((step - head) / one).hex(),
-                                     (one / step).hex()))
+        table.append(f"{(x >> (bits - 63)) + 1 >> 1}ull")
+        x = x * one // root
+    c = (step >> (bits - 99)) + 1 >> 1
+    return ("__device__ const unsigned long long kExp62[4096] = {%s};\nconstexpr unsigned kExpStep2 = %du, "
+            "kExpStep1 = %du, kExpStep0 = %du, kExpPerStep = %du;\n"
+            % (",".join(table), c >> 64, c >> 32 & 0xffffffff, c & 0xffffffff, ((one << 19) + step // 2) // step))
 
 
 def nvcc() -> str:

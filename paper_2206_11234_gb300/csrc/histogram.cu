@@ -11,7 +11,7 @@
 //           key in shared memory (one global atomic per bin and block);
 //   pass 2: each block sorts a tile of ln w by bin in shared memory (counting sort,
 //           integers only), so that a thread adds up consecutive records of one
-//           bin in registers: 16 binary64 instructions per record, and sums leave
+//           bin in registers: 8 binary64 instructions per record, and sums leave
 //           for global memory once per bin change.
 // Bins are right-closed: j = ceil((N - lo)/d) - 1, clamped to [0, n_bins).
 #include <cuda_runtime.h>
@@ -21,7 +21,7 @@
 #include <cstdint>
 #include <cstring>
 
-#include "exp_table.inc"  // kExp64[4096] = 2^(j/4096), kExpStepHi + kExpStepLo = ln 2 / 4096, kExpPerStep its inverse
+#include "exp_table.inc"  // kExp62[4096] = 2^(62 - j/4096), kExpStep2..0 = ln 2 / 4096 x 2^98, kExpPerStep = 4096 / ln 2 x 2^19
 #include "histogram.h"
 
 namespace fpt {
@@ -49,8 +49,10 @@ constexpr long long kSignedNegInf = (long long)0x800fffffffffffffull;
 
 // Fixed point of the bin coordinate: N / d - lo / d + kFix has an ulp of 2^-36.
 constexpr double kFix = 98304.0;  // 1.5 x 2^16
-// largest |edge| / d for which the multiply-add is within 2 ulp (2^-35) of (N - lo) / d
-constexpr double kFastCoord = 8192.0;
+// Largest |edge| / d for which the multiply-add is within 3 ulp of (N - lo) / d:
+// 2^-37 each from its own rounding and fix's (twice that where lo / d = -2^15), 2^-38
+// each from 1/d in both products, 2^-39 from the second's rounding.
+constexpr double kFastCoord = 32768.0;
 
 // Bin of N within its histogram; the comparisons are on integers and the
 // quotient is one multiply-add in fixed point.  Only where that lies within 4 ulp
@@ -163,21 +165,33 @@ __global__ void __launch_bounds__(kMaxThreads) hist_pass_max(const double* __res
     }
 }
 
-// exp(x) for x <= 0 in 8 binary64 instructions: x = k ln 2 / 4096 + r, the table's
-// 2^(k/4096) times the series of exp(r) to r^3, |r| <= 8.5e-5 (table-driven
-// exponential, Tang, ACM TOMS 15 (1989)); within about one unit in the last place.
-// Below -700, infinities and NaN: the library's.
+// exp(x) for x <= 0 in integers (table-driven exponential, Tang, ACM TOMS 15 (1989)):
+// |x| = k ln 2 / 4096 + r in fixed point, the table's 2^(-k/4096) times the series of
+// exp(-r) to r^3, |r| <= 8.5e-5; within 0.77 units in the last place.  Some 50
+// integer instructions take about as long as one of the 8 binary64 instructions that
+// they replace (64 cycles each of a sub-partition): pass 2 of 2^24 records
+// 582 -> 364 us, its binary64 pipe 80 -> 65 % busy, the rest sorting.  From 512 on,
+// infinities and NaN: the library's.
 __device__ __forceinline__ double exp_neg(double x) {
-    if (((unsigned)__double2hiint(x) & 0x7fffffffu) > 0x4085e000u) return exp(x);
-    constexpr double kRound = 6755399441055744.0;  // 1.5 x 2^52
-    const double t = __fma_rn(x, kExpPerStep, kRound);
-    const int k = __double2loint(t);
-    const double kd = __dsub_rn(t, kRound);
-    const double r = __fma_rn(kd, -kExpStepLo, __fma_rn(kd, -kExpStepHi, x));
-    const double p = __fma_rn(__dmul_rn(r, r), __fma_rn(r, 1.0 / 6.0, 0.5), r);
-    const double T = __ldg(&kExp64[k & 4095]);
-    const double e = __fma_rn(T, p, T);
-    return __hiloint2double(__double2hiint(e) + (k >> 12) * (1 << 20), __double2loint(e));
+    const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+    if (hi >= 0x40800000u) return exp(x);
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x)) << 11;
+    const uint64_t z = m >> min(1031 - (int)(hi >> 20), 63);  // |x| 2^55; 0 becomes one unit, too little to matter
+    const uint32_t k = (uint32_t)(((z >> 32) * kExpPerStep + (1ull << 41)) >> 42);
+    const uint64_t kstep = (uint64_t)k * kExpStep1 + __umulhi(k, kExpStep0) + ((uint64_t)(k * kExpStep2) << 32);
+    const int64_t r = (int64_t)((z << 11) - kstep);                   // 2^-66, exact but for the constant, |r| < 2^53
+    const int32_t rs = (int32_t)(r >> 22);                            // 2^-44
+    const uint32_t r2 = (uint32_t)__mulhi(rs, rs);                    // 2^-56
+    const uint32_t w = 0x80000000u - (uint32_t)__mulhi(rs, 174763);   // 1/2 - r/6, 2^-32 (174763 = 2^20 / 6)
+    const int64_t p = r - (int64_t)(((uint64_t)r2 * w) >> 22);        // 1 - exp(-r), 2^-66
+    const uint64_t T = __ldg(&kExp62[k & 4095u]);
+    const int32_t Th = (int32_t)(T >> 32), ph = (int32_t)(p >> 32);
+    const int64_t Tp = (int64_t)Th * ph + __umulhi((uint32_t)Th, (uint32_t)p) +
+                       2 * __mulhi((int32_t)((uint32_t)T >> 1), ph);  // 2^-64
+    uint64_t e = T - (uint64_t)(Tp >> 2);                             // 2^-62, in (1/2, 1 + 1e-4)
+    const uint32_t over = (uint32_t)(e >> 62);
+    e = (e >> over) + 256u;
+    return __longlong_as_double((long long)(((uint64_t)(1021u + over - (k >> 12)) << 52) + (e >> 9)));
 }
 
 constexpr int kSumThreads = 256;  // pass 2
@@ -389,7 +403,9 @@ cudaError_t hist_launch(const HistSeg* d_segs, int n_segs, int max_nb, long long
         N, lw, d_segs, bins, counts, status, bin_idx);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // long runs per thread amortise the last bins' reduction, short ones spread small inputs over the SMs
+    // long runs per thread amortise the sort and the last bins' reduction (2^24 records, 4000 bins: 469 us for
+    // the histogram with 32 per thread, 477 with 20 and 547 with 16, three blocks per SM); short ones spread
+    // small inputs over the SMs
     if (max_n * n_segs >= 4LL * n_sm * kSumThreads * 32)
         e = launch_sum<32>(d_segs, n_segs, max_nb, max_n, lw, bins, n_sm, stream, bin_idx);
     else
