@@ -50,8 +50,8 @@ MLP_MAC_PER_EVAL = 2 * 64 + 64 * 64 + 64
 # for it in profiles/ apply only while their code is unchanged (the C++
 # sources are compared without comments and blank lines; build.py, which
 # holds the compiler flags, as it is).
-STEPPER_SOURCES = ("stepper.cuh", "stepper_f32.cu", "stepper_f64.cu", "stepper_types.h", "rng.cuh", "stepper_launch.h",
-                   "../build.py")
+STEPPER_SOURCES = ("stepper.cuh", "stepper_f32.cuh", "stepper_f32_kahan.cu", "stepper_f32_f64acc.cu", "stepper_f64.cu",
+                   "stepper_types.h", "rng.cuh", "rng64.cuh", "stepper_launch.h", "../build.py")
 
 
 def strip_c_comments(text: str) -> str:
