@@ -516,8 +516,11 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
         }
         if (fixed) break;
     }
-    // up to three chain warps per SM (stepper_few.cuh, with the measurements)
-    if (k.few_func && !fixed && n_total <= 3ull * 32ull * (unsigned long long)n_sm) {
+    // one to few_per_sm chain warps per SM (stepper_few.cuh, with the measurements)
+    if (k.few_func && !fixed && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm)) {
+        int unused = 0;
+        rc = stepper_ctas(k.few_func, kFewThreads, 0, &unused);  // raises the kernel's shared-memory limit
+        if (rc) return rc;
         shape->few = true;
         shape->block = kFewThreads;
         shape->grid = (int)std::max(1ull, (n_total + 31) / 32);

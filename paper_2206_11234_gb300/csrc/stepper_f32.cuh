@@ -20,7 +20,7 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 
 template <int PREC, int MODEL, bool WALL, int FOLD>
 cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
-    stepper_few_kernel<PREC, MODEL, WALL, FOLD><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
+    stepper_few_kernel<float, PREC, MODEL, WALL, FOLD><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -31,7 +31,7 @@ StepperKernel make() {
     if constexpr (MODEL == FPT_MODEL_QUADRATIC || MODEL == kModelPolyLow) {
         k.bench_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD, true>;
         k.bench_launch = &launch<PREC, MODEL, WALL, FOLD, true>;
-        k.few_func = (const void*)stepper_few_kernel<PREC, MODEL, WALL, FOLD>;
+        k.few_func = (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, FOLD>;
         k.few_launch = &launch_few<PREC, MODEL, WALL, FOLD>;
     }
     return k;

@@ -2,6 +2,7 @@
 // FMA contraction off (-fmad=false) so that every operation is rounded exactly
 // as written.
 #include "stepper.cuh"
+#include "stepper_few.cuh"
 #include "stepper_launch.h"
 
 namespace fpt {
@@ -17,9 +18,22 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 }
 
 template <int MODEL, bool WALL, int FOLD>
+cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
+    stepper_few_kernel<double, FPT_PREC_F64, MODEL, WALL, FOLD>
+        <<<grid, block, few_smem_bytes<double, FPT_PREC_F64>(a.n_sets), stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <int MODEL, bool WALL, int FOLD>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, kBlock64, FOLD>,
-                         warp_smem_bytes<double, FPT_PREC_F64>(), &launch<MODEL, WALL, FOLD>};
+    StepperKernel k{(const void*)stepper_kernel<double, FPT_PREC_F64, MODEL, WALL, kBlock64, FOLD>,
+                    warp_smem_bytes<double, FPT_PREC_F64>(), &launch<MODEL, WALL, FOLD>};
+    if constexpr (MODEL == FPT_MODEL_QUADRATIC) {
+        k.few_func = (const void*)stepper_few_kernel<double, FPT_PREC_F64, MODEL, WALL, FOLD>;
+        k.few_per_sm = 4;
+        k.few_launch = &launch_few<MODEL, WALL, FOLD>;
+    }
+    return k;
 }
 
 template <int MODEL, bool WALL>

@@ -14,9 +14,11 @@ struct StepperKernel {
     // the same with runs that take turns (StepperParams::bench > 0), if there is one
     const void* bench_func = nullptr;
     cudaError_t (*bench_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
-    // the stepper for few runs (stepper_few.cuh; blocks of kFewThreads, 32 runs each), if there is one
+    // the stepper for few runs (stepper_few.cuh; blocks of kFewThreads, 32 runs each), if there is one,
+    // and up to how many of its blocks per SM it is the faster
     const void* few_func = nullptr;
     cudaError_t (*few_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
+    int few_per_sm = 3;
 };
 
 inline size_t stepper_smem(const StepperKernel& k, int block, int n_sets, int bench) {

@@ -20,7 +20,7 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 
 template <int PREC, int MODEL, bool WALL>
 cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
-    stepper_few_kernel<PREC, MODEL, WALL, kPowKS><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
+    stepper_few_kernel<float, PREC, MODEL, WALL, kPowKS><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -30,7 +30,7 @@ StepperKernel make() {
                          warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, false>,
                          (const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, true>,
                          &launch<PREC, MODEL, WALL, true>,
-                         (const void*)stepper_few_kernel<PREC, MODEL, WALL, kPowKS>,
+                         (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, kPowKS>,
                          &launch_few<PREC, MODEL, WALL>};
 }
 

@@ -223,3 +223,28 @@ def test_few_runs(nat, kind, n, k_steps):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert out[0][2] == out[1][2]
     assert torch.all(out[0][0][2 * n:2 * n + 5] == 0.0) and torch.all(torch.isinf(out[0][0][2 * n + 5:]))
+
+
+@pytest.mark.parametrize("n", [1, 33, 4097])
+@pytest.mark.parametrize("k_steps", [4, 8])
+def test_few_runs_f64(nat, n, k_steps):
+    """As above for the binary64 mode; walls, and caps at and off the edges of 4, 8 and 16."""
+    import torch
+    base = dict(m=1.0, dN=2e-3, phi_end=1.8)
+    specs = [W.SetSpec(phi_in=2.0, b=0.02, n_traj=n, set_id=1, n_max=3.0, **base),
+             W.SetSpec(phi_in=1.9, b=0.01, n_traj=n, set_id=2, n_max=0.13, phi_uv=1.95, **base),
+             W.SetSpec(phi_in=1.7, b=0.01, n_traj=5, set_id=3, n_max=0.13, **base),
+             W.SetSpec(phi_in=1.9, b=0.0, n_traj=0, set_id=4, n_max=0.13, **base),
+             W.SetSpec(phi_in=4.0, b=0.0, n_traj=n, set_id=5, n_max=0.128, **base)]
+    for some in (specs, specs[:1]):
+        total = sum(s.n_traj for s in some)
+        out = []
+        for block in (0, 128):
+            N = torch.full((total,), -1.0, dtype=torch.float64, device="cuda")
+            lw = torch.full_like(N, -1.0)
+            steps = torch.zeros(1, dtype=torch.int64, device="cuda")
+            p = nat.make_params(m=1.0, n_max=3.0, precision="f64", block_dim=block, k_steps=k_steps, steps_out=steps)
+            nat.fpt_simulate_batch(p, nat.make_sets(some), 12, N, lw)
+            out.append((N, lw, int(steps.item())))
+        assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+        assert out[0][2] == out[1][2]
