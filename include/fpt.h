@@ -98,7 +98,7 @@ typedef struct fpt_params {
     const void* mlp;     /* FPT_BIAS_MLP: device pointer to an fpt_mlp_params */
     int32_t k_eval;      /* FPT_BIAS_MLP: steps between bias evaluations (0 = 32) */
     int32_t block_dim;   /* threads per block of the stepper (0 = autotuned or default) */
-    int32_t k_steps;     /* steps per scheduling block of the stepper (0 = autotuned or default) */
+    int32_t k_steps;     /* steps between two folds of a run's sum of normals (0 = autotuned or default) */
     uint32_t set_id;     /* Philox counter word 3 (fpt_simulate only) */
     uint64_t traj_offset; /* global id of the first trajectory (fpt_simulate only) */
     void* stream;        /* cudaStream_t */
@@ -373,7 +373,7 @@ int fpt_mlp_backward(const fpt_mlp_params* w, const float* phi, const float* N, 
                      float* grad, void* stream);
 
 /* Autotuner of the stepper's launch shape (threads per block in {128, 256, 512}
- * and steps per scheduling block k_steps in {16, 32, 64}, binary64: {4, 8};
+ * and steps per fold k_steps in {16, 32, 64}, binary64: {4, 8};
  * the binary32 power-law bias kernels exist for 32 only).
  * Runs pilot launches over the given sets with each n_traj scaled by
  * `fraction` in (0, 1] (raised if needed so the pilot fills the GPU), times
