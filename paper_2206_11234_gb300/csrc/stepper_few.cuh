@@ -25,6 +25,10 @@
 //
 // Runs are handed out once, 32 to a CTA; all of a warp are at the same step, which
 // is what lets the noise run ahead of them.
+//
+// Every wait ends: a noise warp announces each slot that it was given until it finds the
+// stop flag, and the chain warp, once its runs have finished (at the latest at their cap),
+// takes one more announcement of each slot and gives it back with the flag set.
 #pragma once
 #include "stepper.cuh"
 
