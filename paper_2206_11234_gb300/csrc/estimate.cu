@@ -10,8 +10,10 @@
 //
 // A group of lanes per bin, binary64 throughout: as many lanes as subsets, up to
 // a warp.  What bounds the kernel is the chain of dependent binary64 operations of
-// a bin; the subsets' exponentials and re-centrings are most of it and run side by
-// side (400 bins x 10 subsets: 128 us with one thread per bin and 4 blocks).
+// a bin; the subsets' exponentials and re-centrings run side by side in a group's
+// lanes, the parts of the estimate in the block's warps (EstRole).  400 bins x 10
+// subsets, a call: 128 us with one thread per bin and 4 blocks, 43 with a group of lanes
+// per bin, 33 with a warp per part as well; 60 to 4095 bins without subsets 33 and 19.
 // The group reads the bin's n_sub subset entries, each holding max-shifted sums about its own maximum, and
 // merges them about the common maximum M: s1, s2 rescale by exp(m_k - M), and
 // the moments sum x^r (x = ln w - m_k) re-centre binomially with
@@ -118,20 +120,25 @@ __device__ __forceinline__ double group_max(double v) {
     return v;
 }
 
-constexpr int kEstThreads = 64;
+// What a bin's estimate consists of, a warp of the block each: the parts depend only on
+// the merged sums, which every warp makes for itself.
+enum EstRole { kDirect, kLognormal, kSkew, kKurt, kCumulants, kJackknife, kEstRoles };
 
 template <int G>
-__global__ void __launch_bounds__(kEstThreads)
+__global__ void __launch_bounds__(32 * kEstRoles)
 estimate_kernel(const fpt_bin* __restrict__ bins, int n_bins, int n_sub, double lo, double hi,
                 long long n_total, unsigned long long id_offset, fpt_estimate_bin* __restrict__ out) {
-    const int group = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
-    const int part = (int)(threadIdx.x % G);
+    __shared__ double s_z[2][32];
+    const int role = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
+    const int group = (int)(blockIdx.x * 32 + lane) / G;
+    const int part = lane % G;
     // groups past the last bin work on it too (every lane takes part in the shuffles) and write nothing
     const int j = group < n_bins ? group : n_bins - 1;
     const double d = (hi - lo) / n_bins;
     const double nt = (double)n_total;
     const double qnan = nan("");
-    fpt_estimate_bin o;
+    fpt_estimate_bin& o = out[j];
+    const bool writes = part == 0 && group < n_bins;
     // ---- merge the subsets about the common maximum ----
     double M = -INFINITY;
     for (int k = part; k < n_sub; k += G) {
@@ -161,107 +168,130 @@ estimate_kernel(const fpt_bin* __restrict__ bins, int n_bins, int n_sub, double 
 #pragma unroll
     for (int r = 1; r <= 4; ++r) A.l[r] = group_sum<G>(A.l[r]);
     A.l[0] = A.n;
-    o.count = A.n;
-    // ---- direct / weighted estimate (Eqs. (9), (16)) ----
-    if (A.n > 0.0) {
-        const double e = exp(M);
-        o.p_direct = e * A.s1 / (nt * d);
-        const double v = A.s2 / nt - (A.s1 / nt) * (A.s1 / nt);
-        o.se_direct = e * sqrt(fmax(v, 0.0) / nt) / d;
-    } else {
-        o.p_direct = 0.0;
-        o.se_direct = 0.0;
-    }
-    // ---- lognormal estimate (Eqs. (22)-(24)) ----
-    o.mean_lw = qnan;
-    o.var_lw = qnan;
-    if (A.n == 0.0) {
-        o.p_lognormal = o.eps_lo = o.eps_hi = 0.0;
-    } else if (A.n < 2.0) {
-        o.mean_lw = M + A.l[1] / A.n;
-        o.p_lognormal = o.eps_lo = o.eps_hi = qnan;
-    } else {
-        double mean, var;
-        mean_var(A, &mean, &var);
-        o.mean_lw = M + mean;
-        o.var_lw = var;
-        const double p = A.n * exp(o.mean_lw + 0.5 * var) / (nt * d);
-        const double a = sqrt(var / A.n + var * var / (2.0 * A.n - 2.0));
-        o.p_lognormal = p;
-        o.eps_hi = p * expm1(a);
-        o.eps_lo = -p * expm1(-a);
-    }
-    // ---- D'Agostino-Pearson normality of ln w ----
-    o.skew = o.kurt = o.z_skew = o.z_kurt = o.k2 = o.p_normal = qnan;
-    if (A.n >= 8.0 && o.var_lw > 0.0) {
-        const double n = A.n;
+    const double n = A.n;
+    // central moments, for the parts that use them
+    double m2 = 0.0, m3 = 0.0, m4 = 0.0;
+    if (role == kSkew || role == kKurt || role == kCumulants) {
         const double a1 = A.l[1] / n, a2 = A.l[2] / n, a3 = A.l[3] / n, a4 = A.l[4] / n;
-        const double m2 = a2 - a1 * a1;
-        const double m3 = a3 - 3.0 * a1 * a2 + 2.0 * a1 * a1 * a1;
-        const double m4 = a4 - 4.0 * a1 * a3 + 6.0 * a1 * a1 * a2 - 3.0 * a1 * a1 * a1 * a1;
-        if (m2 > 0.0) {
-            o.skew = m3 / (m2 * sqrt(m2));
-            o.kurt = m4 / (m2 * m2);
-            o.z_skew = skew_z(o.skew, n);
-            o.z_kurt = kurt_z(o.kurt, n);
-            o.k2 = o.z_skew * o.z_skew + o.z_kurt * o.z_kurt;
-            o.p_normal = exp(-0.5 * o.k2);
+        m2 = a2 - a1 * a1;
+        m3 = a3 - 3.0 * a1 * a2 + 2.0 * a1 * a1 * a1;
+        m4 = a4 - 4.0 * a1 * a3 + 6.0 * a1 * a1 * a2 - 3.0 * a1 * a1 * a1 * a1;
+    }
+    if (role == kDirect) {
+        // ---- direct / weighted estimate (Eqs. (9), (16)) ----
+        double p = 0.0, se = 0.0;
+        if (n > 0.0) {
+            const double e = exp(M);
+            p = e * A.s1 / (nt * d);
+            const double v = A.s2 / nt - (A.s1 / nt) * (A.s1 / nt);
+            se = e * sqrt(fmax(v, 0.0) / nt) / d;
         }
-    }
-    // ---- the next cumulant terms of ln <w>: k3/6 + k4/24 (k-statistics) ----
-    o.bias_ln = o.bias_se = qnan;
-    if (A.n >= 4.0 && o.var_lw > 0.0) {
-        const double n = A.n;
-        const double a1 = A.l[1] / n, a2 = A.l[2] / n, a3 = A.l[3] / n, a4 = A.l[4] / n;
-        const double m2 = a2 - a1 * a1;
-        const double m3 = a3 - 3.0 * a1 * a2 + 2.0 * a1 * a1 * a1;
-        const double m4 = a4 - 4.0 * a1 * a3 + 6.0 * a1 * a1 * a2 - 3.0 * a1 * a1 * a1 * a1;
-        if (m2 > 0.0) {
+        if (writes) {
+            o.count = n;
+            o.p_direct = p;
+            o.se_direct = se;
+        }
+    } else if (role == kLognormal) {
+        // ---- lognormal estimate (Eqs. (22)-(24)) ----
+        double mean_lw = qnan, var_lw = qnan, p = 0.0, lo_e = 0.0, hi_e = 0.0;
+        if (n > 0.0 && n < 2.0) {
+            mean_lw = M + A.l[1] / n;
+            p = lo_e = hi_e = qnan;
+        } else if (n > 0.0) {
+            double mean, var;
+            mean_var(A, &mean, &var);
+            mean_lw = M + mean;
+            var_lw = var;
+            p = n * exp(mean_lw + 0.5 * var) / (nt * d);
+            const double a = sqrt(var / n + var * var / (2.0 * n - 2.0));
+            hi_e = p * expm1(a);
+            lo_e = -p * expm1(-a);
+        }
+        if (writes) {
+            o.mean_lw = mean_lw;
+            o.var_lw = var_lw;
+            o.p_lognormal = p;
+            o.eps_lo = lo_e;
+            o.eps_hi = hi_e;
+        }
+    } else if (role == kSkew || role == kKurt) {
+        // ---- D'Agostino-Pearson normality of ln w (m2 > 0: the variance is positive) ----
+        double v = qnan, z = qnan;
+        if (n >= 8.0 && m2 > 0.0) {
+            v = role == kSkew ? m3 / (m2 * sqrt(m2)) : m4 / (m2 * m2);
+            z = role == kSkew ? skew_z(v, n) : kurt_z(v, n);
+        }
+        s_z[role - kSkew][lane] = z;
+        if (writes) {
+            (role == kSkew ? o.skew : o.kurt) = v;
+            (role == kSkew ? o.z_skew : o.z_kurt) = z;
+        }
+    } else if (role == kCumulants) {
+        // ---- the next cumulant terms of ln <w>: k3/6 + k4/24 (k-statistics) ----
+        double bias = qnan, se = qnan;
+        if (n >= 4.0 && m2 > 0.0) {
             const double k2 = n / (n - 1.0) * m2;
             const double k3 = n * n / ((n - 1.0) * (n - 2.0)) * m3;
             const double k4 = n * n * ((n + 1.0) * m4 - 3.0 * (n - 1.0) * m2 * m2) / ((n - 1.0) * (n - 2.0) * (n - 3.0));
             const double v3 = 6.0 * n * k2 * k2 * k2 / ((n - 1.0) * (n - 2.0));
             const double v4 = 24.0 * n * (n + 1.0) * k2 * k2 * k2 * k2 / ((n - 1.0) * (n - 2.0) * (n - 3.0));
-            o.bias_ln = k3 / 6.0 + k4 / 24.0;
-            o.bias_se = sqrt(v3 / 36.0 + v4 / 576.0);
+            bias = k3 / 6.0 + k4 / 24.0;
+            se = sqrt(v3 / 36.0 + v4 / 576.0);
         }
-    }
-    // ---- jackknife over the subsets (§2.1) ----
-    o.jk_direct = o.jk_lognormal = qnan;
-    if (n_sub >= 2) {
-        // a lane's first subset estimate is kept for the second sum (all of them up to 32 subsets)
-        double sd = 0.0, sl = 0.0, pd0 = 0.0, pl0 = 0.0;
-        for (int k = part; k < n_sub; k += G) {
-            const BinSums s = load_bin(bins[(long long)k * n_bins + j]);
-            const double tk = subset_total(n_total, id_offset, n_sub, k);
-            const double pd = tk > 0.0 ? direct_p(s, tk, d) : qnan;
-            const double pl = tk > 0.0 ? lognormal_p(s, tk, d) : qnan;
-            if (k == part) {
-                pd0 = pd;
-                pl0 = pl;
-            }
-            sd += pd;
-            sl += pl;
+        if (writes) {
+            o.bias_ln = bias;
+            o.bias_se = se;
         }
-        const double md = group_sum<G>(sd) / n_sub, ml = group_sum<G>(sl) / n_sub;
-        double vd = 0.0, vl = 0.0;
-        for (int k = part; k < n_sub; k += G) {
-            double pd = pd0, pl = pl0;
-            if (k != part) {
+    } else {
+        // ---- jackknife over the subsets (§2.1) ----
+        double jd = qnan, jl = qnan;
+        if (n_sub >= 2) {
+            // a lane's first subset estimate is kept for the second sum (all of them up to 32 subsets)
+            double sd = 0.0, sl = 0.0, pd0 = 0.0, pl0 = 0.0;
+            for (int k = part; k < n_sub; k += G) {
                 const BinSums s = load_bin(bins[(long long)k * n_bins + j]);
                 const double tk = subset_total(n_total, id_offset, n_sub, k);
-                pd = tk > 0.0 ? direct_p(s, tk, d) : qnan;
-                pl = tk > 0.0 ? lognormal_p(s, tk, d) : qnan;
+                const double pd = tk > 0.0 ? direct_p(s, tk, d) : qnan;
+                const double pl = tk > 0.0 ? lognormal_p(s, tk, d) : qnan;
+                if (k == part) {
+                    pd0 = pd;
+                    pl0 = pl;
+                }
+                sd += pd;
+                sl += pl;
             }
-            vd += (pd - md) * (pd - md);
-            vl += (pl - ml) * (pl - ml);
+            const double md = group_sum<G>(sd) / n_sub, ml = group_sum<G>(sl) / n_sub;
+            double vd = 0.0, vl = 0.0;
+            for (int k = part; k < n_sub; k += G) {
+                double pd = pd0, pl = pl0;
+                if (k != part) {
+                    const BinSums s = load_bin(bins[(long long)k * n_bins + j]);
+                    const double tk = subset_total(n_total, id_offset, n_sub, k);
+                    pd = tk > 0.0 ? direct_p(s, tk, d) : qnan;
+                    pl = tk > 0.0 ? lognormal_p(s, tk, d) : qnan;
+                }
+                vd += (pd - md) * (pd - md);
+                vl += (pl - ml) * (pl - ml);
+            }
+            vd = group_sum<G>(vd);
+            vl = group_sum<G>(vl);
+            jd = sqrt(vd / (n_sub - 1)) / sqrt((double)n_sub);
+            jl = sqrt(vl / (n_sub - 1)) / sqrt((double)n_sub);
         }
-        vd = group_sum<G>(vd);
-        vl = group_sum<G>(vl);
-        o.jk_direct = sqrt(vd / (n_sub - 1)) / sqrt((double)n_sub);
-        o.jk_lognormal = sqrt(vl / (n_sub - 1)) / sqrt((double)n_sub);
+        if (writes) {
+            o.jk_direct = jd;
+            o.jk_lognormal = jl;
+        }
     }
-    if (part == 0 && group < n_bins) out[j] = o;
+    __syncthreads();
+    if (role == kSkew) {
+        const double k2 = s_z[0][lane] * s_z[0][lane] + s_z[1][lane] * s_z[1][lane];
+        const double p = exp(-0.5 * k2);
+        if (writes) {
+            o.k2 = k2;
+            o.p_normal = p;
+        }
+    }
 }
 
 // ---- multi-bias reconstruction: inverse-variance combination in log space ----
@@ -448,8 +478,8 @@ extern "C" int fpt_estimate(const fpt_bin* bins, int32_t n_bins, int32_t n_sub, 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     auto launch = [&](auto lanes) {
         constexpr int G = decltype(lanes)::value;
-        const int per_block = kEstThreads / G;
-        estimate_kernel<G><<<(n_bins + per_block - 1) / per_block, kEstThreads, 0, st>>>(
+        const int per_block = 32 / G;
+        estimate_kernel<G><<<(n_bins + per_block - 1) / per_block, 32 * kEstRoles, 0, st>>>(
             bins, n_bins, n_sub, lo, hi, (long long)n_total, id_offset, out);
     };
     if (n_sub == 1) launch(std::integral_constant<int, 1>{});
