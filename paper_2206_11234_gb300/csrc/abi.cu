@@ -62,8 +62,8 @@ cudaError_t lib_malloc_from_pool_async(void** p, size_t bytes, cudaMemPool_t poo
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
-// The library's stream-ordered memory pool, one per device, created on first
-// use, for the allocations made afresh at every call (call workspaces, the
+// The library's stream-ordered memory pool, one per device (pools belong to the
+// device and outlive its contexts), created on first use, for the allocations made afresh at every call (call workspaces, the
 // host-buffer entry's device buffers).  Its release threshold is the maximum,
 // so what one call frees stays mapped for the next; the default pool returns
 // memory to the system at every synchronisation, and mapping tens or hundreds
@@ -425,9 +425,10 @@ int pick_stepper(const fpt_params* p, bool wall, StepperKernel* k, int* block) {
     return FPT_OK;
 }
 
-// CTAs of a stepper that fit on one SM, by the occupancy API; kept per kernel and
-// shape (the answer is the kernel's alone), since a query costs a small call more
-// than a microsecond.
+// CTAs of a stepper that fit on one SM, by the occupancy API; kept per device, kernel
+// and shape, since a query costs a small call more than a microsecond.  So is the
+// raised shared-memory limit: the runtime keeps kernels and their attributes per
+// device, for every context there is or will be (tests/test_gpu_context_change.py).
 static int stepper_ctas(const void* func, int block, size_t smem, int* per_sm) {
     static std::mutex mu;
     static std::map<std::tuple<int, const void*, int, size_t>, int> cache;
