@@ -314,6 +314,12 @@ static void expected_length(const fpt_params* p, const SetConst& c, double* step
     *spread = std::sqrt(var) / c.dN;
 }
 
+// A run's steps to the end of its last block of q: lengths that spread over blocks end
+// in the middle of one on average.
+static double padded_length(double steps, double spread, double q) {
+    return spread < 0.25 * q ? q * std::ceil((steps + 1.0) / q) : steps + 0.5 * q;
+}
+
 void order_tickets(const fpt_params* p, SetConst* table, const fpt_set* sets, int n_sets, RunLengths* len) {
     struct Item {
         double steps, spread;
@@ -321,13 +327,15 @@ void order_tickets(const fpt_params* p, SetConst* table, const fpt_set* sets, in
         int set;
     };
     std::vector<Item> order(n_sets);
-    *len = RunLengths{0.0, 0.0, 0.0};
+    *len = RunLengths{};
     for (int i = 0; i < n_sets; ++i) {
         order[i].n = (long long)sets[i].n_traj;
         order[i].set = i;
         expected_length(p, table[i], &order[i].steps, &order[i].spread);
         len->total += order[i].steps * (double)order[i].n;
         if (order[i].n > 0) len->longest = std::fmax(len->longest, order[i].steps);
+        for (int q = 0; q < 3 && order[i].steps > 0.0; ++q)
+            len->padded[q] += padded_length(order[i].steps, order[i].spread, 16 << q) * (double)order[i].n;
     }
     std::stable_sort(order.begin(), order.end(), [](const Item& a, const Item& b) { return a.steps > b.steps; });
     // the tickets handed out last decide how long the launch trails off
@@ -478,6 +486,15 @@ static double step_cycles(double warps) { return std::fmax(49.0 + 16.0 * warps, 
 // per scheduler, and the launch takes the time of three.  Fewer warps that take
 // turns at a few more runs each (StepperParams::bench) even that out.
 //
+// Brief runs (binary32).  A run occupies its lane to the end of a scheduling block.
+// Blocks of 64 steps take 8 to 12 % less time per step than those of one fold, but
+// where runs are short that is lost again (2^22 runs, us, blocks of 16 and 64):
+// 12 steps 251 365, 44 steps 313 364, 60 steps 366 365, 80 steps 527 554, 200 steps
+// 845 949, 300 steps 1155 1120.  They keep all resident warps, which hide what starting
+// and ending a run costs (320,000 runs of 12 steps 58 us, 66 with half).  The general polynomial spills in the longer block,
+// which matters where the SMs are full: 40,000 runs 173 172, 100,000 289 300, 300,000
+// 624 674, 2,000,000 3292 3567.
+//
 // Threads per block (0: free): the largest block whose CTAs load every SM alike
 // (40,000 runs are 157 CTAs of 256 threads, two of them on five of the 152 SMs:
 // 6.08 ms; as 128-thread CTAs 4.82 ms).
@@ -495,15 +512,18 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
     const bool uneven = len.longest * (double)n_total > 1.5 * len.total;
     int best = 0;
     shape->bench = 0;
+    const bool brief = k.brief_func && 1.12 * len.padded[k.fold <= 16 ? 0 : 1] < len.padded[2];
+    shape->brief = brief || (k.brief_func && n_total > 32ull * k.brief_warps * (unsigned long long)n_sm);
+    const void* func = shape->brief ? k.brief_func : k.func;
     for (int b = fixed ? fixed : first; b >= 32; b >>= 1) {
         int per_sm = 0;
-        rc = stepper_ctas(k.func, b, stepper_smem(k, b, n_sets, 0), &per_sm);
+        rc = stepper_ctas(func, b, stepper_smem(k, b, n_sets, 0), &per_sm);
         if (rc) return rc;
         const int warps = b / 32, full = per_sm * warps;
         int r = full;
         const double trail = share > 0.0 ? len.tail * full / share : 0.0;
-        if (trail > 0.15) r = full / 2;
-        else if (trail > 0.06) r = 3 * full / 4;
+        if (trail > 0.15 && !brief) r = full / 2;
+        else if (trail > 0.06 && !brief) r = 3 * full / 4;
         if (uneven) r = std::min(r, std::max(8, (int)std::ceil(1.25 * share / len.longest)));
         per_sm = std::max(1, r / warps);
         const unsigned long long need = std::max(1ull, (n_total + b - 1) / b);
@@ -523,11 +543,12 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
         rc = stepper_ctas(k.few_func, kFewThreads, 0, &unused);  // raises the kernel's shared-memory limit
         if (rc) return rc;
         shape->few = true;
+        shape->brief = false;
         shape->block = kFewThreads;
         shape->grid = (int)std::max(1ull, (n_total + 31) / 32);
         return FPT_OK;
     }
-    if (!k.bench_func || uneven || !(len.tail <= 0.1 * len.longest)) return FPT_OK;
+    if (shape->brief || !k.bench_func || uneven || !(len.tail <= 0.1 * len.longest)) return FPT_OK;
     const int b = fixed ? fixed : 128, warps = b / 32;
     int per_sm = 0;
     rc = stepper_ctas(k.bench_func, b, stepper_smem(k, b, n_sets, 32), &per_sm);
@@ -622,7 +643,11 @@ int enqueue_run(const fpt_params* p, const Prepared& P, const WorkspaceLayout& L
     a.n_sm = shape.n_sm;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
     if (P.n_total > 0) {
-        cudaError_t e = (shape.few ? k.few_launch : shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
+        const auto launch = shape.few         ? k.few_launch
+                            : shape.bench > 0 ? k.bench_launch
+                            : shape.brief     ? k.brief_launch
+                                              : k.launch;
+        cudaError_t e = launch(a, shape.grid, shape.block, stream);
         if (e != cudaSuccess) return cuda_fail(e, "stepper launch");
     }
     if (after_stepper) {

@@ -43,10 +43,12 @@ int check_params(const fpt_params* p);
 // since the occupancy API is conservative for kernels that allocate TMEM.
 int resident_ctas(const void* func, int threads, size_t dyn_smem, int tmem_cols, int* per_sm);
 
-// Expected lengths of the runs of a launch, in steps: their sum, the longest set
-// and how far runs of the sets handed out last may outlast their expectation.
+// Expected lengths of the runs of a launch, in steps: their sum, the longest set,
+// how far runs of the sets handed out last may outlast their expectation, and the
+// sum with each run taken to the end of a block of 16, 32 or 64 steps.
 struct RunLengths {
     double total, longest, tail;
+    double padded[3];
 };
 constexpr long long kTrailingRuns = 1 << 17;  // about the lanes of one GPU
 
@@ -88,6 +90,7 @@ struct LaunchShape {
     int bench = 0;            // runs that take turns with each warp's 32 ...
     int bench_every = 0;      // ... every so many scheduling blocks
     bool few = false;         // the stepper for few runs
+    bool brief = false;       // scheduling blocks of one fold
     int n_sm = 1;
 };
 int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsigned long long n_total,

@@ -154,7 +154,11 @@ extern "C" int fpt_simulate_batch_noalloc(const fpt_params* p, const fpt_set* se
     a.bench_every = shape.bench_every;
     a.n_sm = shape.n_sm;
     a.steps_out = reinterpret_cast<unsigned long long*>(p->steps_out);
-    e = (shape.few ? k.few_launch : shape.bench > 0 ? k.bench_launch : k.launch)(a, shape.grid, shape.block, stream);
+    const auto launch = shape.few         ? k.few_launch
+                        : shape.bench > 0 ? k.bench_launch
+                        : shape.brief     ? k.brief_launch
+                                          : k.launch;
+    e = launch(a, shape.grid, shape.block, stream);
     if (e != cudaSuccess) return cuda_fail(e, "stepper launch");
 
     StepperScratch host;

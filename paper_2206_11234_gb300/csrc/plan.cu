@@ -116,7 +116,8 @@ extern "C" int fpt_plan_create(const fpt_params* p, const fpt_set* sets, int32_t
             if (cudaGraphNodeGetType(nodes[i], &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
             cudaKernelNodeParams kp;
             if (cudaGraphKernelNodeGetParams(nodes[i], &kp) != cudaSuccess) continue;
-            if (kp.func == k.func || (k.bench_func && kp.func == k.bench_func) || (k.few_func && kp.func == k.few_func)) {
+            if (kp.func == k.func || (k.bench_func && kp.func == k.bench_func) || (k.few_func && kp.func == k.few_func) ||
+                (k.brief_func && kp.func == k.brief_func)) {
                 pl->stepper_node = nodes[i];
                 pl->knp = kp;
                 std::memcpy(&pl->sp, kp.kernelParams[0], sizeof(StepperParams));

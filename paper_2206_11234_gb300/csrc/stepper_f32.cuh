@@ -10,11 +10,11 @@ namespace {
 
 constexpr int kBlock32 = 64;  // steps of a scheduling block, whatever k_steps folds
 
-template <int PREC, int MODEL, bool WALL, int FOLD, bool BENCH>
+template <int PREC, int MODEL, bool WALL, int FOLD, bool BENCH, int KS = kBlock32>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) +
                         (size_t)(block / 32) * (warp_smem_bytes<float, PREC>() + a.bench * kParkWords * 4);
-    stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD, BENCH><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<float, PREC, MODEL, WALL, KS, FOLD, BENCH><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -33,6 +33,12 @@ StepperKernel make() {
         k.bench_launch = &launch<PREC, MODEL, WALL, FOLD, true>;
         k.few_func = (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, FOLD>;
         k.few_launch = &launch_few<PREC, MODEL, WALL, FOLD>;
+    }
+    if constexpr (FOLD < kBlock32) {
+        k.brief_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, FOLD, FOLD, false>;
+        k.brief_launch = &launch<PREC, MODEL, WALL, FOLD, false, FOLD>;
+        k.fold = FOLD;
+        if (MODEL == FPT_MODEL_POLYNOMIAL) k.brief_warps = 16;
     }
     return k;
 }

@@ -19,6 +19,12 @@ struct StepperKernel {
     const void* few_func = nullptr;
     cudaError_t (*few_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
     int few_per_sm = 3;
+    // the same in scheduling blocks of one fold, for brief runs, if there is one, and from how many
+    // warps per SM on it is the faster whatever the runs' length
+    const void* brief_func = nullptr;
+    int fold = 0;  // steps of its block
+    unsigned long long brief_warps = 1ull << 40;
+    cudaError_t (*brief_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
 };
 
 inline size_t stepper_smem(const StepperKernel& k, int block, int n_sets, int bench) {

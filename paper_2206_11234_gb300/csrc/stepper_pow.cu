@@ -10,11 +10,11 @@ namespace {
 
 constexpr int kPowKS = 32;
 
-template <int PREC, int MODEL, bool WALL, bool BENCH>
+template <int PREC, int MODEL, bool WALL, bool BENCH, int KS = 2 * kPowKS>
 cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     const size_t smem = stepper_table_bytes(a.n_sets) +
                         (size_t)(block / 32) * (warp_smem_bytes<float, PREC>() + a.bench * kParkWords * 4);
-    stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, BENCH><<<grid, block, smem, stream>>>(a);
+    stepper_kernel<float, PREC, MODEL, WALL, KS, kPowKS, BENCH><<<grid, block, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -26,12 +26,16 @@ cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t
 
 template <int PREC, int MODEL, bool WALL>
 StepperKernel make() {
-    return StepperKernel{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, false>,
-                         warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, false>,
-                         (const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, true>,
-                         &launch<PREC, MODEL, WALL, true>,
-                         (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, kPowKS>,
-                         &launch_few<PREC, MODEL, WALL>};
+    StepperKernel k{(const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, false>,
+                    warp_smem_bytes<float, PREC>(), &launch<PREC, MODEL, WALL, false>};
+    k.bench_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, 2 * kPowKS, kPowKS, true>;
+    k.bench_launch = &launch<PREC, MODEL, WALL, true>;
+    k.few_func = (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, kPowKS>;
+    k.few_launch = &launch_few<PREC, MODEL, WALL>;
+    k.brief_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, kPowKS, kPowKS, false>;
+    k.brief_launch = &launch<PREC, MODEL, WALL, false, kPowKS>;
+    k.fold = kPowKS;
+    return k;
 }
 
 template <int PREC, bool WALL>

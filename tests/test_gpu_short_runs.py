@@ -1,0 +1,83 @@
+"""Runs of a few to a few hundred steps: the launch that the library picks for them
+gives the records of the one for long runs, and is not the slower one.
+
+The times compare two launches of one call on the same box, best of many
+passes; the faults they were written for were 1.3 to 1.5 times as slow.
+"""
+import math
+
+import pytest
+
+from paper_2206_11234_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nat(cuda_device):
+    from paper_2206_11234_gb300 import native
+    return native
+
+
+def spec(steps, n, **kw):
+    """Runs of about `steps` steps: the classical duration from phi = 2 is 1/2."""
+    return W.SetSpec(**{**dict(phi_in=2.0, m=0.1, b=0.3, dN=0.5 / steps, n_max=4.0, n_traj=n), **kw})
+
+
+def batch(nat, specs, **kw):
+    import torch
+    n = sum(s.n_traj for s in specs)
+    N = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+    lw = torch.full_like(N, -1.0)
+    p = nat.make_params(m=specs[0].m, n_max=4.0, **kw)
+    sets = nat.make_sets(specs)
+    return lambda: (nat.fpt_simulate_batch(p, sets, 3, N, lw), N, lw)[1:]
+
+
+def best_us(f, passes=30):
+    import torch
+    f()
+    out = []
+    for _ in range(passes):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        out.append(1e3 * a.elapsed_time(b))
+    return min(out)
+
+
+KINDS = {"f32_kahan": dict(precision="f32_kahan"), "f32_f64acc": dict(precision="f32_f64acc"),
+         "power": dict(precision="f32_kahan", bias_p=3.0), "power_real": dict(precision="f32_f64acc", bias_p=2.5),
+         "constant": dict(precision="f32_kahan", model=1, a0=-0.6, s0=0.05),
+         "quartic": dict(precision="f32_f64acc", model=2, poly=[0, 0, 0, 0, 0.01]),
+         "general": dict(precision="f32_kahan", model=2, poly=[0, 0, 0.1, 0, 0, 0, 1e-4])}
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("k_steps", [16, 32])
+@pytest.mark.parametrize("steps", [1, 15, 16, 17, 40])
+def test_short_runs_have_the_records_they_have_beside_long_ones(nat, kind, k_steps, steps):
+    """Alone, and in a call whose other runs are long: the same records, bit for bit,
+    with a wall, caps at and off block edges, and runs that start past their end."""
+    import torch
+    kw = dict(KINDS[kind])
+    if not kind.startswith("power"):
+        kw["k_steps"] = k_steps
+    b = 1e-3 if kind.startswith("power") else 0.3
+    short = [spec(steps, 20011, b=b, set_id=1), spec(steps, 3001, b=b, set_id=2, phi_uv=2.02, n_max=0.5),
+             spec(steps, 77, b=b, set_id=3, phi_in=1.3), spec(steps, 1, b=b, set_id=4, n_max=0.01)]
+    long = spec(2000, 30000, b=b, set_id=5)
+    N, lw = batch(nat, short, **kw)()
+    N2, lw2 = batch(nat, short + [long], **kw)()
+    n = N.numel()
+    assert torch.equal(N, N2[:n]) and torch.equal(lw, lw2[:n])
+    assert torch.all(N[20011 + 3001:-1] == 0.0)
+
+
+@pytest.mark.parametrize("precision", ["f32_kahan", "f32_f64acc"])
+def test_short_runs_do_not_pay_for_long_blocks(nat, precision):
+    """Blocks of 64 steps (k_steps = 64 has no others) take 365 us for these, blocks of 16 251."""
+    s = [spec(12, 1 << 22)]
+    assert best_us(batch(nat, s, precision=precision)) < 0.85 * best_us(batch(nat, s, precision=precision, k_steps=64))
