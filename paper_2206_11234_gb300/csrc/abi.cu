@@ -484,7 +484,11 @@ static double step_cycles(double warps) { return std::fmax(49.0 + 16.0 * warps, 
 // Bench (binary32).  Runs of one length that are not a whole number of waves leave
 // some schedulers with one warp more than the others: 40,000 runs are 2.06 warps
 // per scheduler, and the launch takes the time of three.  Fewer warps that take
-// turns at a few more runs each (StepperParams::bench) even that out.
+// turns at a few more runs each (StepperParams::bench) even that out.  Filling and
+// emptying the bench costs as much as some 1000 steps per warp of a scheduler, so
+// shorter runs do without (us without and with turns, runs of 500, 1000, 2000, 4000
+// steps): 40,000 runs 67 72, 92 92, 133 131, 227 194; 60,000 69 82, 106 108, 166 158,
+// 289 255; 160,000 109 132, 179 203, 314 353, 573 576.
 //
 // Brief runs (binary32).  A run occupies its lane to the end of a scheduling block.
 // Blocks of 64 steps take 8 to 12 % less time per step than those of one fold, but
@@ -548,13 +552,15 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
         shape->grid = (int)std::max(1ull, (n_total + 31) / 32);
         return FPT_OK;
     }
-    if (shape->brief || !k.bench_func || uneven || !(len.tail <= 0.1 * len.longest)) return FPT_OK;
+    const double x = (double)n_total / (128.0 * n_sm);  // warps per scheduler, if all ran at once
+    if (shape->brief || !k.bench_func || uneven || !(len.tail <= 0.1 * len.longest) ||
+        len.longest < std::fmax(2500.0, 1000.0 * x))
+        return FPT_OK;
     const int b = fixed ? fixed : 128, warps = b / 32;
     int per_sm = 0;
     rc = stepper_ctas(k.bench_func, b, stepper_smem(k, b, n_sets, 32), &per_sm);
     if (rc) return rc;
     // waves of all warps that fit, and a rest: the time of a step of every run
-    const double x = (double)n_total / (128.0 * n_sm);  // warps per scheduler, if all ran at once
     const double k_full = best / 4.0;
     const double waves = std::floor(x / k_full + 1e-9);
     double time = waves * step_cycles(k_full) + (x > waves * k_full ? step_cycles(std::ceil(x - waves * k_full)) : 0.0);

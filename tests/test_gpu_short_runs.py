@@ -81,3 +81,34 @@ def test_short_runs_do_not_pay_for_long_blocks(nat, precision):
     """Blocks of 64 steps (k_steps = 64 has no others) take 365 us for these, blocks of 16 251."""
     s = [spec(12, 1 << 22)]
     assert best_us(batch(nat, s, precision=precision)) < 0.85 * best_us(batch(nat, s, precision=precision, k_steps=64))
+
+
+@pytest.mark.parametrize("kind", ["f32_kahan", "power"])
+def test_short_runs_do_not_take_turns(nat, kind):
+    """Three per cent more runs than eight warps per scheduler: with turns runs of 300 steps took
+    1.4 times as long as those of the whole waves."""
+    import torch
+    whole = torch.cuda.get_device_properties(0).multi_processor_count * 128 * 8
+    b = 1e-3 if kind == "power" else 0.0
+    t = [best_us(batch(nat, [spec(300, n, m=0.01, b=b)], **KINDS[kind])) for n in (whole, whole * 103 // 100)]
+    assert t[1] < 1.2 * t[0], t
+
+
+@pytest.mark.parametrize("kind", ["f32_kahan", "f32_f64acc", "power", "quartic"])
+@pytest.mark.parametrize("n", [20011, 24000, 40001, 60000])
+@pytest.mark.parametrize("phi_uv", [math.inf, 2.0])
+def test_long_runs_that_take_turns(nat, kind, n, phi_uv):
+    """Run counts just above a whole number of warps per scheduler, 4000 to 5000 steps
+    of one length, with and without a wall: the records of calls of 4096 runs by their
+    offsets, bit for bit."""
+    import torch
+    kw = dict(KINDS[kind])
+    if kind == "quartic":
+        kw["poly"] = [0, 0, 0, 0, 1e-7]
+    base = dict(phi_in=2.0, m=0.01, dN=1e-4, b=1e-3, phi_uv=phi_uv, set_id=4,
+                n_max=0.4 if n == 24000 else 1.0, phi_end=1.8 if kind == "quartic" else W.PHI_END)
+    N, lw = batch(nat, [W.SetSpec(n_traj=n, **base)], **kw)()
+    for off in range(0, n, 4096):
+        k = min(4096, n - off)
+        N1, l1 = batch(nat, [W.SetSpec(n_traj=k, traj_offset=off, **base)], **kw)()
+        assert torch.equal(N[off:off + k], N1) and torch.equal(lw[off:off + k], l1), off
