@@ -541,8 +541,10 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
         }
         if (fixed) break;
     }
-    // one to few_per_sm chain warps per SM (stepper_few.cuh, with the measurements)
-    if (k.few_func && !fixed && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm)) {
+    // one to few_per_sm chain warps per SM (stepper_few.cuh, with the measurements); a run of less than some
+    // 48 steps is done before the noise warps are of use (14,000 binary64 runs of 12 steps: 45 us without, 66 with)
+    if (k.few_func && !fixed && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm) &&
+        len.total >= 48.0 * (double)n_total) {
         int unused = 0;
         rc = stepper_ctas(k.few_func, kFewThreads, 0, &unused);  // raises the kernel's shared-memory limit
         if (rc) return rc;

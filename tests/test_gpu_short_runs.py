@@ -112,3 +112,10 @@ def test_long_runs_that_take_turns(nat, kind, n, phi_uv):
         k = min(4096, n - off)
         N1, l1 = batch(nat, [W.SetSpec(n_traj=k, traj_offset=off, **base)], **kw)()
         assert torch.equal(N[off:off + k], N1) and torch.equal(lw[off:off + k], l1), off
+
+
+def test_few_short_binary64_runs(nat):
+    """14,000 binary64 runs of 12 steps: 45 us in the persistent stepper (a caller's
+    block_dim keeps it), 66 with separate noise warps."""
+    s = [spec(12, 14000)]
+    assert best_us(batch(nat, s, precision="f64")) < 1.2 * best_us(batch(nat, s, precision="f64", block_dim=64))
