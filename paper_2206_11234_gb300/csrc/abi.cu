@@ -541,18 +541,20 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
         }
         if (fixed) break;
     }
-    // one to few_per_sm chain warps per SM (stepper_few.cuh, with the measurements); a run of less than some
-    // 48 steps is done before the noise warps are of use (14,000 binary64 runs of 12 steps: 45 us without, 66 with)
+    // one to few_per_sm chain warps per SM, all at once (stepper_few.cuh, with the measurements); a run of less than
+    // some 48 steps is done before the noise warps are of use (14,000 binary64 runs of 12 steps: 45 us without, 66 with)
     if (k.few_func && !fixed && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm) &&
         len.total >= 48.0 * (double)n_total) {
-        int unused = 0;
-        rc = stepper_ctas(k.few_func, kFewThreads, 0, &unused);  // raises the kernel's shared-memory limit
+        int per_sm = 0;
+        rc = stepper_ctas(k.few_func, kFewThreads, stepper_table_bytes(n_sets) + k.few_smem, &per_sm);
         if (rc) return rc;
-        shape->few = true;
-        shape->brief = false;
-        shape->block = kFewThreads;
-        shape->grid = (int)std::max(1ull, (n_total + 31) / 32);
-        return FPT_OK;
+        if (n_total <= 32ull * (unsigned long long)(per_sm * n_sm)) {
+            shape->few = true;
+            shape->brief = false;
+            shape->block = kFewThreads;
+            shape->grid = (int)std::max(1ull, (n_total + 31) / 32);
+            return FPT_OK;
+        }
     }
     const double x = (double)n_total / (128.0 * n_sm);  // warps per scheduler, if all ran at once
     if (shape->brief || !k.bench_func || uneven || !(len.tail <= 0.1 * len.longest) ||

@@ -20,7 +20,7 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 
 template <int PREC, int MODEL, bool WALL, int FOLD>
 cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
-    stepper_few_kernel<float, PREC, MODEL, WALL, FOLD><<<grid, block, few_smem_bytes<float, PREC>(a.n_sets), stream>>>(a);
+    stepper_few_kernel<float, PREC, MODEL, WALL, FOLD><<<grid, block, stepper_table_bytes(a.n_sets) + few_smem_bytes<float, PREC>(), stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -32,6 +32,7 @@ StepperKernel make() {
         k.bench_func = (const void*)stepper_kernel<float, PREC, MODEL, WALL, kBlock32, FOLD, true>;
         k.bench_launch = &launch<PREC, MODEL, WALL, FOLD, true>;
         k.few_func = (const void*)stepper_few_kernel<float, PREC, MODEL, WALL, FOLD>;
+        k.few_smem = few_smem_bytes<float, PREC>();
         k.few_launch = &launch_few<PREC, MODEL, WALL, FOLD>;
     }
     if constexpr (FOLD < kBlock32) {

@@ -20,7 +20,7 @@ cudaError_t launch(const StepperParams& a, int grid, int block, cudaStream_t str
 template <int MODEL, bool WALL, int FOLD>
 cudaError_t launch_few(const StepperParams& a, int grid, int block, cudaStream_t stream) {
     stepper_few_kernel<double, FPT_PREC_F64, MODEL, WALL, FOLD>
-        <<<grid, block, few_smem_bytes<double, FPT_PREC_F64>(a.n_sets), stream>>>(a);
+        <<<grid, block, stepper_table_bytes(a.n_sets) + few_smem_bytes<double, FPT_PREC_F64>(), stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -31,6 +31,7 @@ StepperKernel make() {
     if constexpr (MODEL == FPT_MODEL_QUADRATIC) {
         k.few_func = (const void*)stepper_few_kernel<double, FPT_PREC_F64, MODEL, WALL, FOLD>;
         k.few_per_sm = 4;
+        k.few_smem = few_smem_bytes<double, FPT_PREC_F64>();
         k.few_launch = &launch_few<MODEL, WALL, FOLD>;
     }
     return k;

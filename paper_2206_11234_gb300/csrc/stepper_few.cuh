@@ -39,20 +39,23 @@ static_assert(kFewThreads == 32 * (1 + kNoiseWarps), "one chain warp and its noi
 
 // what a step pair needs of its noise, [slot][part][pair][lane]
 //   binary32: {t0, t1, rho, c + s} with step terms t, or {q c, q s} with the power bias
-//   binary64: {t0, t1}, {r, c}, {s}
+//   binary64: {t0, t1}, {r, c}, and s in an array of its own behind them, so that four CTAs of
+//   64 sets fit on an SM (padded to a third part they were three, and 19,456 runs took a second
+//   wave: 2585 -> 2175 us, with a wall 1768 -> 1160; persistent stepper 2960 and 1326)
 template <typename Real>
 struct FewNoise {
     using Part = float4;
-    static constexpr int kParts = 1;
+    static constexpr int kParts = 1, kSingles = 0;
 };
 template <>
 struct FewNoise<double> {
     using Part = double2;
-    static constexpr int kParts = 3;
+    static constexpr int kParts = 2, kSingles = 1;
 };
 template <typename Real>
-constexpr size_t kRingBytes =
-    (size_t)kNoiseWarps * FewNoise<Real>::kParts * 8 * 32 * sizeof(typename FewNoise<Real>::Part);
+constexpr size_t kRingBytes = (size_t)kNoiseWarps * 8 * 32 *
+                              (FewNoise<Real>::kParts * sizeof(typename FewNoise<Real>::Part) +
+                               FewNoise<Real>::kSingles * sizeof(Real));
 
 // Hand-over of a slot between its noise warp and the chain warp, 64 threads each:
 // one side arrives and goes on, the other waits for it.
@@ -67,9 +70,10 @@ __device__ __forceinline__ void hand_wait(int id) {
 __device__ __forceinline__ int full_id(int slot) { return 1 + slot; }
 __device__ __forceinline__ int empty_id(int slot) { return 1 + kNoiseWarps + slot; }
 
+// dynamic shared memory but for the set table
 template <typename Real, int PREC>
-constexpr size_t few_smem_bytes(int n_sets) {
-    return stepper_table_bytes(n_sets) + kRingBytes<Real> + 32 * sizeof(Pending<Real, PREC>);
+constexpr int few_smem_bytes() {
+    return (int)(kRingBytes<Real> + 32 * sizeof(Pending<Real, PREC>));
 }
 
 template <typename Real, int PREC, int MODEL, bool WALL, int FOLD>
@@ -86,6 +90,7 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
     SetConst* s_sets = reinterpret_cast<SetConst*>(s_dyn);
     long long* s_first = reinterpret_cast<long long*>(s_dyn + (size_t)n_sets * sizeof(SetConst));
     Part* ring = reinterpret_cast<Part*>(s_dyn + stepper_table_bytes(n_sets));
+    Real* singles = reinterpret_cast<Real*>(ring + kNoiseWarps * kSlot);  // binary64 only
     Entry* q = reinterpret_cast<Entry*>(s_dyn + stepper_table_bytes(n_sets) + kRingBytes<Real>);
     for (int i = threadIdx.x; i < n_sets; i += blockDim.x) {
         s_sets[i] = P.sets[i];
@@ -122,6 +127,7 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
             uint32_t V[12];
             philox_group(pl, G, P.keys, V);
             Part f[kSlot / 32];
+            [[maybe_unused]] Real single[8];
 #pragma unroll
             for (int p = 0; p < 8; ++p) {
                 if constexpr (F64) {
@@ -129,7 +135,7 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
                     const double q2 = __dmul_rn(np.r, model.kq);
                     f[p] = make_double2(__fma_rn(q2, np.c, model.tc), __fma_rn(q2, np.s, model.tc));
                     f[8 + p] = make_double2(np.r, np.c);
-                    f[16 + p] = make_double2(np.s, 0.0);
+                    single[p] = np.s;
                 } else {
                     const NormalPair np = group_pair_f32(V, p >> 1, p & 1);
                     const float q2 = __fmul_rn(model.kq, np.rho);
@@ -146,6 +152,10 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
             }
 #pragma unroll
             for (int p = 0; p < kSlot / 32; ++p) out[32 * p] = f[p];
+            if constexpr (F64) {
+#pragma unroll
+                for (int p = 0; p < 8; ++p) singles[slot * 256 + 32 * p + lane] = single[p];
+            }
             hand_arrive(full_id(slot));
         }
     }
@@ -194,7 +204,7 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
 #pragma unroll
             for (int p = 0; p < 8; ++p) {
                 const double2 t = f[32 * p], rc = f[32 * (8 + p)];
-                const double s = f[32 * (16 + p)].x;
+                const double s = singles[slot * 256 + 32 * p + lane];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     phi = model.step(phi, h == 0 ? t.x : t.y);

@@ -19,6 +19,7 @@ struct StepperKernel {
     const void* few_func = nullptr;
     cudaError_t (*few_launch)(const StepperParams&, int grid, int block, cudaStream_t stream) = nullptr;
     int few_per_sm = 3;
+    int few_smem = 0;  // dynamic shared memory of a block but for the set table
     // the same in scheduling blocks of one fold, for brief runs, if there is one, and from how many
     // warps per SM on it is the faster whatever the runs' length
     const void* brief_func = nullptr;

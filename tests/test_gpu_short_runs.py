@@ -119,3 +119,17 @@ def test_few_short_binary64_runs(nat):
     block_dim keeps it), 66 with separate noise warps."""
     s = [spec(12, 14000)]
     assert best_us(batch(nat, s, precision="f64")) < 1.2 * best_us(batch(nat, s, precision="f64", block_dim=64))
+
+
+def test_few_binary64_runs_of_64_sets(nat):
+    """As many binary64 runs as the stepper with separate noise warps takes, in as many
+    sets as a call may have: its CTAs hold all their tables at once.  The records of
+    the persistent stepper, and not in more time (two waves took 1.33 times as long)."""
+    import torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 128
+    sets = [W.SetSpec(phi_in=3.0, m=0.1, b=1.0, dN=1e-3, n_max=4.0, phi_uv=3.0, set_id=i,
+                      n_traj=n // 64 + (i < n % 64)) for i in range(64)]
+    f, g = batch(nat, sets, precision="f64"), batch(nat, sets, precision="f64", block_dim=64)
+    for x, y in zip(f(), g()):
+        assert torch.equal(x, y)
+    assert best_us(f, 10) < 1.1 * best_us(g, 10)
