@@ -97,7 +97,7 @@ typedef struct fpt_params {
     double poly[FPT_POLY_TERMS]; /* FPT_MODEL_POLYNOMIAL: coefficients of V (the sets' m is ignored) */
     const void* mlp;     /* FPT_BIAS_MLP: device pointer to an fpt_mlp_params */
     int32_t k_eval;      /* FPT_BIAS_MLP: steps between bias evaluations (0 = 32) */
-    int32_t block_dim;   /* threads per block of the stepper (0 = autotuned or default) */
+    int32_t block_dim;   /* threads per block of the persistent stepper (0 = autotuned or default) */
     int32_t k_steps;     /* steps between two folds of a run's sum of normals (0 = autotuned or default) */
     uint32_t set_id;     /* Philox counter word 3 (fpt_simulate only) */
     uint64_t traj_offset; /* global id of the first trajectory (fpt_simulate only) */
@@ -379,7 +379,8 @@ int fpt_mlp_backward(const fpt_mlp_params* w, const float* phi, const float* N, 
  * `fraction` in (0, 1] (raised if needed so the pilot fills the GPU), times
  * each shape with CUDA events on p->stream and keeps the fastest in EM steps
  * per second.  The result is cached per (device, precision, model, wall) and
- * used by every later call whose block_dim or k_steps is 0.  Outputs (host,
+ * used by every later call whose block_dim or k_steps is 0; the block is the
+ * persistent stepper's, calls of few runs keep their own.  Outputs (host,
  * each may be NULL): the chosen shape and its pilot steps/s.  Records do not
  * depend on block_dim; k_steps only changes the rounding of the ln w sum. */
 int fpt_autotune(const fpt_params* p, const fpt_set* sets, int32_t n_sets, uint64_t seed,

@@ -501,7 +501,10 @@ static double step_cycles(double warps) { return std::fmax(49.0 + 16.0 * warps, 
 //
 // Threads per block (0: free): the largest block whose CTAs load every SM alike
 // (40,000 runs are 157 CTAs of 256 threads, two of them on five of the 152 SMs:
-// 6.08 ms; as 128-thread CTAs 4.82 ms).
+// 6.08 ms; as 128-thread CTAs 4.82 ms).  The autotuner's block holds for this kernel
+// alone, which is what it measured: the stepper for few runs and the turns are taken
+// with it as without (32 runs of 40,000 steps 0.70 ms, 1.03 in one block of 512); only a
+// caller's own block_dim keeps them off.
 int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsigned long long n_total,
                  const RunLengths& len, LaunchShape* shape) {
     int n_sm = 0;
@@ -543,7 +546,7 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
     }
     // one to few_per_sm chain warps per SM, all at once (stepper_few.cuh, with the measurements); a run of less than
     // some 48 steps is done before the noise warps are of use (14,000 binary64 runs of 12 steps: 45 us without, 66 with)
-    if (k.few_func && !fixed && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm) &&
+    if (k.few_func && p->block_dim == 0 && n_total <= 32ull * (unsigned long long)(k.few_per_sm * n_sm) &&
         len.total >= 48.0 * (double)n_total) {
         int per_sm = 0;
         rc = stepper_ctas(k.few_func, kFewThreads, stepper_table_bytes(n_sets) + k.few_smem, &per_sm);
@@ -560,7 +563,7 @@ int stepper_grid(const fpt_params* p, const StepperKernel& k, int n_sets, unsign
     if (shape->brief || !k.bench_func || uneven || !(len.tail <= 0.1 * len.longest) ||
         len.longest < std::fmax(2500.0, 1000.0 * x))
         return FPT_OK;
-    const int b = fixed ? fixed : 128, warps = b / 32;
+    const int b = p->block_dim ? p->block_dim : 128, warps = b / 32;
     int per_sm = 0;
     rc = stepper_ctas(k.bench_func, b, stepper_smem(k, b, n_sets, 32), &per_sm);
     if (rc) return rc;
