@@ -275,17 +275,18 @@ int make_set_const(const fpt_params* p, const fpt_set& s, long long first, SetCo
 
 // Expected length of a run of the set and its spread, in steps: the noise-free
 // duration, the integral of dphi / |D + B|, and the small-noise standard
-// deviation, the square root of the integral of S^2 / |D + B|^3 dphi, by the
-// midpoint rule; at most the censoring cap, which is also taken (with no spread)
-// where the biased drift does not point down.
+// deviation, the square root of the integral of S^2 / |D + B|^3 dphi, by four
+// Gauss–Legendre nodes (64 sets cost a call 3 us; 16 midpoints cost it 8, for more
+// error); at most the censoring cap, which is also taken (with no spread) where the
+// biased drift does not point down.
 static void expected_length(const fpt_params* p, const SetConst& c, double* steps, double* spread) {
-    constexpr int kNodes = 16;
+    constexpr double kNode[4] = {0.06943184420297371, 0.33000947820757187, 0.6699905217924281, 0.9305681557970263};
+    constexpr double kWeight[4] = {0.17392742256872693, 0.32607257743127307, 0.32607257743127307, 0.17392742256872693};
     *steps = *spread = 0.0;
     if (!(c.phi_in > c.phi_end)) return;
-    const double h = (c.phi_in - c.phi_end) / kNodes;
     double dur = 0.0, var = 0.0;
-    for (int i = 0; i < kNodes; ++i) {
-        const double x = c.phi_end + (i + 0.5) * h;
+    for (int i = 0; i < 4; ++i) {
+        const double x = c.phi_end + kNode[i] * (c.phi_in - c.phi_end), h = kWeight[i] * (c.phi_in - c.phi_end);
         double D, S;
         if (p->model == FPT_MODEL_CONSTANT) {
             D = c.a0;
@@ -307,8 +308,9 @@ static void expected_length(const fpt_params* p, const SetConst& c, double* step
             *steps = (double)c.m_max;
             return;
         }
-        dur += h / v;
-        var += h * S * S / (v * v * v);
+        const double t = h / v;
+        dur += t;
+        var += t * S * S / (v * v);
     }
     *steps = std::fmin(dur / c.dN, (double)c.m_max);
     *spread = std::sqrt(var) / c.dN;
