@@ -1,8 +1,10 @@
 """Calls on little data: the launches chosen for them, at the edges of their ranges, and their
 times against calls of the same box (best of many; the faults they were written for were
 1.2 to 1.6 times as slow)."""
+import numpy as np
 import pytest
 
+import oracle
 from paper_2206_11234_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -43,3 +45,36 @@ def test_many_sets_cost_little_on_the_host(nat):
         return lambda: nat.fpt_simulate_batch(p, sets, 3, N, lw)
 
     assert best_us(call(64)) < 1.3 * best_us(call(1))
+
+
+@pytest.mark.parametrize("n_bins,n_sub", [(1, 1), (3, 1), (5, 1), (1021, 1), (1025, 1), (4096, 1), (64, 64), (7, 3)])
+@pytest.mark.parametrize("size", [1, 2, 255, 256, 257, 8192, "wave", "wave+1"])
+def test_histograms_of_few_records(nat, n_bins, n_sub, size):
+    """Counts and maxima exactly, sums to rounding (as the larger ones), with one
+    record per thread up to a CTA per SM and eight from there on."""
+    import torch
+    wave = 256 * torch.cuda.get_device_properties(0).multi_processor_count
+    n = {"wave": wave, "wave+1": wave + 1}.get(size, size)
+    N, lw = W.random_records(n, seed=n_bins, lo=0.0, hi=6.0)
+    bins, counts = nat.empty_bins(n_bins * n_sub), nat.empty_counts(1)
+    nat.fpt_histogram(torch.from_numpy(N).cuda(), torch.from_numpy(lw).cuda(), n_bins, 0.0, 6.0, bins, counts, n_sub=n_sub,
+                      id_offset=5)
+    ref, ref_counts = oracle.histogram(N, lw, n_bins, 0.0, 6.0, n_sub=n_sub, id_offset=5)
+    ref, got = ref.reshape(-1, 8), bins.cpu().numpy()
+    assert np.array_equal(counts.cpu().numpy()[0], ref_counts)
+    assert np.array_equal(got.view(np.int64)[:, 7], ref[:, 7].astype(np.int64))
+    assert np.array_equal(got[:, 0], ref[:, 0])
+    np.testing.assert_allclose(got[:, 1:7], ref[:, 1:7], rtol=1e-12, atol=1e-300)
+
+
+def test_many_bins_cost_few_records_little(nat):
+    """100 records into 4096 bins and into one: calls of 57 and 46 us with eight records
+    per thread and a bin per thread of the scan."""
+    import torch
+    N, lw = (torch.from_numpy(x).cuda() for x in W.random_records(100, seed=1, lo=0.0, hi=6.0))
+
+    def call(nb):
+        bins, counts = nat.empty_bins(nb), nat.empty_counts(1)
+        return lambda: nat.fpt_histogram(N, lw, nb, 0.0, 6.0, bins, counts)
+
+    assert best_us(call(4096)) < 1.13 * best_us(call(1))
