@@ -9,6 +9,7 @@
 //   dW1 += d1 x^T, db1 += d1
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "abi_internal.h"
@@ -95,6 +96,12 @@ constexpr uint32_t kIdescDW2 = tc::idesc_bf16_tn(128, 64, true, true);   // delt
 // and 320 shuffles per row and tile, and 56 KB of copies, so that three CTAs fit
 // where two did.  1,000,003 rows: 280 us with them, 150 us without, 139 us with two
 // threads per row (24 warps per SM instead of 12).
+//
+// CTAs.  Each ends with 4489 additions to the one gradient, some 0.1 us that the CTAs
+// take in turn: fewer of them are the faster until an SM has enough tiles for two or
+// three (calls in us with 1, 2 and 3 per SM: 20,000 rows 58 61 60, 58,368 60 85 101,
+// 100,000 64 75 98, 300,000 97 98 111, 600,000 135 123 133, 1,000,000 195 160 161,
+// 4,000,000 615 447 408).
 constexpr int kBwdThreads = 256;  // two threads per row, 32 of the 64 units each
 
 __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_mlp_params* __restrict__ P,
@@ -305,10 +312,12 @@ __global__ void __launch_bounds__(kBwdThreads, 3) mlp_backward_kernel(const fpt_
     }
 }
 
+constexpr int kMaxCtas = 32;  // per SM: no limit but the kernel's own
+
 // Grid for a persistent MLP kernel and a check that its resident CTAs cannot
 // ask for more TMEM columns than an SM has (an allocation would then wait for
 // a CTA that never exits).
-int mlp_grid(const void* func, int threads, size_t smem, int tmem_cols, long long tiles, int* grid) {
+int mlp_grid(const void* func, int threads, size_t smem, int tmem_cols, long long tiles, int max_per_sm, int* grid) {
     int n_sm = 0;
     int rc = device_sm_count(&n_sm);
     if (rc) return rc;
@@ -318,7 +327,7 @@ int mlp_grid(const void* func, int threads, size_t smem, int tmem_cols, long lon
     rc = resident_ctas(func, threads, smem, tmem_cols, &per_sm);
     if (rc) return rc;
     if (per_sm < 1) return fail(FPT_EUNSUPPORTED, "MLP kernel does not fit on an SM");
-    const long long full = (long long)per_sm * n_sm;
+    const long long full = (long long)std::min(per_sm, max_per_sm) * n_sm;
     *grid = (int)(tiles < full ? (tiles < 1 ? 1 : tiles) : full);
     return FPT_OK;
 }
@@ -399,7 +408,7 @@ extern "C" int fpt_mlp_forward(const fpt_mlp_params* w, const float* phi, const 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t smem = mlp_fwd_smem_bytes();
     int grid = 0;
-    int rc = mlp_grid((const void*)mlp_forward_kernel, 128, smem, kFwdTmemCols, (n + 127) / 128, &grid);
+    int rc = mlp_grid((const void*)mlp_forward_kernel, 128, smem, kFwdTmemCols, (n + 127) / 128, kMaxCtas, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
     cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
@@ -424,7 +433,12 @@ extern "C" int fpt_mlp_backward(const fpt_mlp_params* w, const float* phi, const
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t smem = sizeof(MlpBwdSmem);
     int grid = 0;
-    int rc = mlp_grid((const void*)mlp_backward_kernel, kBwdThreads, smem, kBwdTmemCols, (n + 127) / 128, &grid);
+    const long long tiles = (n + 127) / 128;
+    int n_sm = 0;
+    int rc = device_sm_count(&n_sm);
+    if (rc) return rc;
+    rc = mlp_grid((const void*)mlp_backward_kernel, kBwdThreads, smem, kBwdTmemCols, tiles,
+                  tiles < 20LL * n_sm ? 1 : tiles < 50LL * n_sm ? 2 : kMaxCtas, &grid);
     if (rc) return rc;
     unsigned* d_status = nullptr;
     cudaError_t e = lib_malloc_retained_async(reinterpret_cast<void**>(&d_status), sizeof(unsigned), st);
