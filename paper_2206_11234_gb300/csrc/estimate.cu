@@ -13,7 +13,8 @@
 // a bin; the subsets' exponentials and re-centrings run side by side in a group's
 // lanes, the parts of the estimate in the block's warps (EstRole).  400 bins x 10
 // subsets, a call: 128 us with one thread per bin and 4 blocks, 43 with a group of lanes
-// per bin, 33 with a warp per part as well; 60 to 4095 bins without subsets 33 and 19.
+// per bin, 33 with a warp per part as well; 60 to 4095 bins without subsets 33 and 19;
+// 2048 bins x 2 subsets 56, 60 with eight lanes per bin and 19 with two.
 // The group reads the bin's n_sub subset entries, each holding max-shifted sums about its own maximum, and
 // merges them about the common maximum M: s1, s2 rescale by exp(m_k - M), and
 // the moments sum x^r (x = ln w - m_k) re-centre binomially with
@@ -483,6 +484,7 @@ extern "C" int fpt_estimate(const fpt_bin* bins, int32_t n_bins, int32_t n_sub, 
             bins, n_bins, n_sub, lo, hi, (long long)n_total, id_offset, out);
     };
     if (n_sub == 1) launch(std::integral_constant<int, 1>{});
+    else if (n_sub == 2) launch(std::integral_constant<int, 2>{});
     else if (n_sub <= 8) launch(std::integral_constant<int, 8>{});
     else launch(std::integral_constant<int, 32>{});
     const cudaError_t e = cudaGetLastError();
