@@ -7,7 +7,7 @@ namespace fpt {
 constexpr unsigned kStatusWaitExpired = 1u;   // a bounded tensor-core wait gave up
 // set only by the bounds checks of an FPT_DEBUG build, which then skip the access:
 constexpr unsigned kStatusSetIndex = 0x10u;   // a ticket's parameter set does not hold its record
-constexpr unsigned kStatusQueueFull = 0x20u;  // a warp's replay queue would overflow
+constexpr unsigned kStatusQueueFull = 0x20u;  // a warp's replay queue or its bench would overflow
 constexpr unsigned kStatusRecord = 0x40u;     // a record index at or beyond the run total
 constexpr unsigned kStatusHistBin = 0x80u;    // a histogram bin index beyond the edge clamp
 

@@ -763,9 +763,18 @@ stepper_kernel(const StepperParams P) {
                 if (filling) {
                     // the bench's runs, not yet started, leave the lanes
                     const unsigned on = __ballot_sync(FULL, live);
+#if FPT_DEBUG
+                    if (__popc(on) > P.bench) {
+                        atomicOr(&P.scratch->status, kStatusQueueFull);
+                        live = live && __popc(on & lt_mask) < P.bench;  // the others are dropped, not written
+                    }
+#endif
                     if (live) save(bench_slot + __popc(on & lt_mask), P.bench);
                     live = false;
                     waiting = __popc(on);
+#if FPT_DEBUG
+                    if (waiting > P.bench) waiting = P.bench;
+#endif
                     until = P.bench_every;
                     filling = false;
                     __syncwarp();

@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
         s_sets[i] = P.sets[i];
         s_first[i] = P.sets[i].ticket0;
     }
+    if (threadIdx.x == 0) s_first[n_sets] = (long long)P.n_total;
     if (threadIdx.x < kNoiseWarps) s_stop[threadIdx.x] = 0;
     __syncthreads();
 
@@ -107,12 +108,18 @@ __global__ void __launch_bounds__(kFewThreads) stepper_few_kernel(const StepperP
 
     // this lane's run: ticket 32 blockIdx + lane, the last set s with ticket0[s] <= ticket
     const unsigned long long t = 32ull * blockIdx.x + lane;
-    const bool have = t < P.n_total;
+    bool have = t < P.n_total;
     int lo = 0, hi = n_sets - 1;
     while (have && lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if ((long long)t >= s_first[mid]) lo = mid; else hi = mid - 1;
     }
+#if FPT_DEBUG
+    if (have && ((long long)t < s_first[lo] || (long long)t >= s_first[lo + 1])) {
+        atomicOr(&P.scratch->status, kStatusSetIndex);
+        have = false;  // as if there were no such run
+    }
+#endif
     const SetConst& S = s_sets[lo];
     const unsigned long long i = have ? t - (unsigned long long)s_first[lo] : 0ull;
     typename StepOf<Real, MODEL>::type model;
