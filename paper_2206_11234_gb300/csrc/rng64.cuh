@@ -14,7 +14,10 @@
 //     -2 ln u0 = n 2 ln 2 + 2 ln(2 inv) - 2 ln(1 - r'/2), the last term as its series
 //     to r'^5.  Near u0 = 1 the entry is 1/2 and both constants vanish, so the
 //     result keeps its relative accuracy there;
-//   * sqrt by one third-order step from the hardware's reciprocal square root.
+//   * the root and the reciprocal by one third-order step from the hardware's seeds:
+//     Householder's iteration of the second order (Householder, The Numerical
+//     Treatment of a Single Nonlinear Equation (1970)), for 1/x the geometric series
+//     of 1/(1 - e) to e^2, for the root the binomial series of (1 - e)^(-1/2) to e^2.
 // Against 80-bit arithmetic of the same angles the radius errs by 5.2e-17 on
 // average and 2.9e-16 at most, the cosine by half a unit in the last place.
 // The tables are written at build time (build.py) in exact integer arithmetic.
