@@ -63,8 +63,9 @@ cudaError_t lib_malloc_from_pool_async(void** p, size_t bytes, cudaMemPool_t poo
 }
 
 // The library's stream-ordered memory pool, one per device (pools belong to the
-// device and outlive its contexts), created on first use, for the allocations made afresh at every call (call workspaces, the
-// host-buffer entry's device buffers).  Its release threshold is the maximum,
+// device and outlive its contexts), created on first use, for the allocations made
+// afresh at every call (call workspaces, the scratch of the network and training
+// entries, the host-buffer entry's device buffers).  Its release threshold is the maximum,
 // so what one call frees stays mapped for the next; the default pool returns
 // memory to the system at every synchronisation, and mapping tens or hundreds
 // of megabytes again costs milliseconds per call.
@@ -496,10 +497,11 @@ static double step_cycles(double warps) { return std::fmax(49.0 + 16.0 * warps, 
 // Blocks of 64 steps take 8 to 12 % less time per step than those of one fold, but
 // where runs are short that is lost again (2^22 runs, us, blocks of 16 and 64):
 // 12 steps 251 365, 44 steps 313 364, 60 steps 366 365, 80 steps 527 554, 200 steps
-// 845 949, 300 steps 1155 1120.  They keep all resident warps, which hide what starting
-// and ending a run costs (320,000 runs of 12 steps 58 us, 66 with half).  The general polynomial spills in the longer block,
-// which matters where the SMs are full: 40,000 runs 173 172, 100,000 289 300, 300,000
-// 624 674, 2,000,000 3292 3567.
+// 845 949, 300 steps 1155 1120.  They keep all resident warps,
+// which hide what starting and ending a run costs (320,000 runs of 12 steps 58 us, 66
+// with half).  The general polynomial (eight coefficients) gains nothing from the longer
+// block, and where the SMs are full loses by it, whatever its runs' length (40,000 runs 173 172,
+// 100,000 289 300, 300,000 624 674, 2,000,000 3292 3567; both spill some 40 bytes).
 //
 // Threads per block (0: free): the largest block whose CTAs load every SM alike
 // (40,000 runs are 157 CTAs of 256 threads, two of them on five of the 152 SMs:

@@ -121,18 +121,13 @@ __device__ __forceinline__ void mlp_issue_z2(MlpTile& S) {
     tc::mma_commit(&S.mbar);
 }
 
-// All threads: publish this thread's operand writes, let thread 0 issue the
-// MMAs of `issue` and commit them, wait for the commit (bounded).
-template <class Issue>
-__device__ __forceinline__ void mlp_tile_mma(MlpTile& S, uint32_t& phase, Issue issue) {
+// All threads: publish this thread's operand writes, let thread 0 issue z2,
+// wait for its commit (bounded).
+__device__ __forceinline__ void mlp_tile_z2(MlpTile& S, uint32_t& phase) {
     tc::fence_before_sync();
     tc::fence_proxy_async();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        tc::fence_after_sync();
-        issue();
-        tc::mma_commit(&S.mbar);
-    }
+    if (threadIdx.x == 0) mlp_issue_z2(S);
     if (S.status != 0u || !tc::mbar_wait(&S.mbar, phase)) S.status = 1u;  // one expiry, not one per tile
     phase ^= 1u;
     tc::fence_after_sync();
@@ -149,13 +144,7 @@ __device__ __forceinline__ float mlp_tile_forward(MlpTile& S, float phi, float N
     const float x1 = (N - S.norm[2]) * S.norm[3];
     mlp_layer1_to_tile<8, WIDE ? 8 : 1>(S, S.A, tid, x0, x1);
     // z2 = W2 h1 (b2 is added below)
-    mlp_tile_mma(S, phase, [&] {
-        const uint32_t a = tc::smem_u32(S.A), w2 = tc::smem_u32(S.W2);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)  // K = 64 in steps of 16 (two core matrices = 256 bytes)
-            tc::mma_bf16(S.tmem, tc::smem_desc(a + 256 * kk, 128, 1024), tc::smem_desc(w2 + 256 * kk, 128, 1024),
-                         kIdescZ2, kk > 0 ? 1u : 0u);
-    });
+    mlp_tile_z2(S, phase);
     // h2 = tanh(z2 + b2) in BF16 (two units per MUFU operation), b = w3 . h2 + b3
     const uint32_t taddr = S.tmem + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16);
     float b = S.b3;

@@ -4,13 +4,13 @@
 // normals) lives in registers.  Lanes advance in scheduling blocks of KS
 // steps with no per-step control flow: each step is the biased EM update of
 // §2.2 Eq. (11) followed by the reflecting wall, and the lane keeps the
-// minimum phi of the block.  At the block end a lane whose minimum reached
-// phi_end (first passage, §2.1 below Eq. (8)) or whose step count reached the
-// censoring cap has finished somewhere inside the block: it pushes its
-// block-start state onto its warp's replay queue in shared memory and refills
+// minimum phi of the block.  Every FOLD steps a run that has neither reached
+// phi_end (first passage, §2.1 below Eq. (8)) nor the censoring cap commits its
+// state.  At the block end a lane whose run has finished somewhere inside pushes
+// the state last committed onto its warp's replay queue in shared memory and refills
 // at once from a global ticket counter (one atomicAdd per warp), so a warp
 // keeps 32 live runs whatever their lengths (persistent scheduler).  When 32
-// finished runs are queued, the warp replays their blocks together, step by
+// finished runs are queued, the warp replays their folds together, step by
 // step with a test after each step — bit-identical arithmetic, the same
 // Philox counters — to find the exact step, interpolates the crossing time in
 // binary64 and writes the records.  Replays thus run with all 32 lanes busy
@@ -112,10 +112,9 @@ struct ModelStep<float, FPT_MODEL_CONSTANT> {
 // D = -V'/V and S = sqrt(V) / (2 pi sqrt 3), and the step is
 // dphi = S t + D dN with t = b dN + sqrt(dN) xi (so the bias is B = b S).  The
 // coefficients are read from the set table in shared memory.  DEGREE: Horner's
-// rule starts at c_DEGREE; leading out the zero coefficients above it changes
-// no bit (0 phi + c = c), and the degree-4
-// kernel keeps its coefficients in registers: 100,003 runs of phi^4 in 296
-// instead of 356 us.
+// rule starts at c_DEGREE; leaving out the zero coefficients above it changes
+// no bit (0 phi + c = c), and the degree-4 kernel keeps its coefficients in
+// registers: 100,003 runs of phi^4 in 296 instead of 356 us.
 template <int DEGREE>
 struct PolyStep {
     float tc, kq, dN;   // tc = b dN, kq = -sqrt(2 ln 2) sqrt(dN), dN
@@ -641,18 +640,19 @@ __device__ __forceinline__ void replay_batch(const Pending<Real, PREC>* q, int c
 // the kernel, 64-step blocks): 64 registers, 512 threads (32 warps per SM):
 // 1.335e12; 56 registers, 384 threads (36 warps): 1.325e12; 48 registers,
 // 256 threads (40 warps): 1.313e12 -- more resident warps do not pay for the
-// spills they need.  At 64 the quadratic, constant and
-// power-law kernels are spill-free; the polynomial-potential ones (eight
-// coefficients per set) spill 12-48 bytes (56-84 at a cap of 56).  The binary64
-// reference kernels are built with a larger cap.
+// spills they need.  At 64 the quadratic, constant and power-law kernels spill 0 to
+// 24 bytes, the polynomial-potential ones (five or eight coefficients per set) 12 to
+// 72.  The binary64 reference kernels are built with a larger cap.
+//
+// KS: steps of a scheduling block.  FOLD: the sum of the normals is folded into the
+// running sum W every FOLD steps; that sets the rounding of ln w, so it is what a
+// caller's k_steps chooses, while the block length is free (64 steps in binary32, or
+// one fold for brief runs: stepper_grid in abi.cu; 16 steps in binary64).
+// BENCH: with runs that take turns (StepperParams::bench); for at most 16 warps per
+// SM, so with twice the registers (at 64 the turns' state cost the step 4-14 %).
 #ifndef FPT_STEPPER_MAXNREG
 #define FPT_STEPPER_MAXNREG 64
 #endif
-//
-// KS: steps of a scheduling block.  FOLD: the sum of the normals is folded into the running sum W every FOLD steps; that sets the rounding of ln w,
-// so it is what a caller's k_steps chooses, while the block length is free.
-// BENCH: with runs that take turns (StepperParams::bench); for at most 16 warps per
-// SM, so with twice the registers (at 64 the turns' state cost the step 4-14 %).
 template <typename Real, int PREC, int MODEL, bool WALL, int KS, int FOLD, bool BENCH = false>
 __global__ void __maxnreg__(BENCH ? 128 : FPT_STEPPER_MAXNREG)
 stepper_kernel(const StepperParams P) {
