@@ -96,20 +96,20 @@ def stepper_source_hash() -> str:
 def stepper_counters(precision, block_dim, k_steps, name="stepper_counters.json"):
     """The ncu counters recorded for a stepper kernel in profiles/ (DRAM bytes,
     instructions, pipe activity, branch and lane efficiency of one launch over
-    a stated number of runs and steps), or None when no record matches this
-    kernel's precision, launch shape (threads per block and block length) and
-    source."""
+    a stated number of runs and steps), or None when none of the file's records
+    matches this kernel's precision, launch shape (threads per block and steps per
+    fold) and source."""
     path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "profiles", name)
     try:
         with open(path) as fh:
-            rec = json.load(fh)
+            recs = json.load(fh)
     except (OSError, ValueError):
         return None
-    if (rec.get("precision"), rec.get("block_dim"), rec.get("k_steps")) != (precision, block_dim, k_steps):
-        return None
-    if rec.get("source_sha256") != stepper_source_hash():
-        return None
-    return rec
+    for rec in recs if isinstance(recs, list) else [recs]:
+        if ((rec.get("precision"), rec.get("block_dim"), rec.get("k_steps")) == (precision, block_dim, k_steps)
+                and rec.get("source_sha256") == stepper_source_hash()):
+            return rec
+    return None
 
 
 def parse():
