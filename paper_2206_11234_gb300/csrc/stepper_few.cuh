@@ -7,18 +7,21 @@
 // scoreboards.  Here the chain is alone in its warp: the noise warps, on the SM's
 // other schedulers, write what a step needs of each Box–Muller pair to shared
 // memory, every third 16-step group each, and the chain warp reads it one group
-// ahead: 28 cycles per step and some 90 per group for the hand-over.  The numbers,
-// their order and so the records are those of the persistent stepper, bit for bit.
+// ahead: 28 cycles per step and some 50 to 90 per group for the hand-over, 31 to 33 cycles
+// per step alone on an SM (39 with binary64 sums, 41 to 47 with a wall, 42 to 57 with three
+// on an SM).  The numbers, their order and so the records are those of the persistent
+// stepper, bit for bit.
 // us, persistent -> this, at one and at three chain warps per SM (4864, 14,592 runs):
-// power 2423 -> 1783, 2409 -> 2206; wall 3891 -> 2903, 3862 -> 3455; ladder
-// 293 -> 232, 279 -> 263; quartic 151 -> 110, 137 -> 119; diffusive 1057 -> 917 at
-// three; 512 runs to N = 1 156 -> 116.  With four per SM the noise warps contend with the
+// power 2423 -> 1783, 2409 -> 2206; wall 3784 -> 2801, 3782 -> 3403; ladder
+// 258 -> 183, 256 -> 233; quartic 151 -> 110, 137 -> 119; diffusive 1057 -> 917 at
+// three; 512 runs of some 2150 steps 146 -> 109.  With four per SM the noise warps contend with the
 // chains (0.93 to 1.19 times as fast), with six they lose (0.71 to 1.0).
 // Slots of two groups read without the copy ahead measured 3 to 9 % slower.
 //
 // Binary64 (quadratic model).  A warp has the binary64 unit of its scheduler, one
 // instruction per 64 cycles, 15 per step: 9 of them are noise, which the noise warps
 // take to the other schedulers' units; 6 are left to the chain.
+// 516 cycles per step alone on an SM, 720 with a wall, 772 and 945 with three.
 // us, persistent -> this: 500 runs 2119 -> 1073 (m = 1, to N = 6), 9728 2671 -> 1422,
 // 16,384 2994 -> 2253, 19,456 2985 -> 2211; with a wall, m = 0.1, 19,456 2718 -> 2321;
 // with a fifth CTA on an SM (24,320) 3153 -> 3076 and 3051 -> 3978.
