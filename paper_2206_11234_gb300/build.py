@@ -28,7 +28,9 @@ LIB = os.path.join(HERE, "libfpt_gb300.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
+# Device code uncompressed: a unit is unpacked as a whole at its first call, which cost a process 15 ms
+# for a binary32 stepper and 11 ms for the binary64 one (a library of 29 MB; 92 without).
+COMMON = ["-O3", "-lineinfo", "--no-compress", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
 UNITS = {
     "abi.cu": [],
     "histogram.cu": [],

@@ -21,10 +21,15 @@
 // Against 80-bit arithmetic of the same angles the radius errs by 5.2e-17 on
 // average and 2.9e-16 at most, the cosine by half a unit in the last place.
 // The tables are written at build time (build.py) in exact integer arithmetic.
+//
+// A translation unit without binary64 kernels defines FPT_NO_F64 first, which keeps
+// the tables out: 1 MB of device memory per unit, and 5 ms of its first call.
 #pragma once
 #include <cstdint>
 
+#ifndef FPT_NO_F64
 #include "f64_tables.inc"  // bits of kTrig64[65536] {cos, sin}, kLog64[1024] {-2 inv, 2 ln(2 inv)}, kLn2N64[33] = n 2 ln 2
+#endif
 #include "rng.cuh"
 
 namespace fpt {
@@ -32,6 +37,11 @@ namespace fpt {
 struct PairF64 {
     double r, c, s;  // normals r c, r s
 };
+
+#ifdef FPT_NO_F64
+__device__ PairF64 pair_f64(uint32_t rad, uint32_t h);
+__device__ PairF64 group_pair_f64(const uint32_t V[12], int j, int p);
+#endif
 
 __device__ __forceinline__ double2 table_pair(const ulonglong2* t) {
     const ulonglong2 v = __ldg(t);
@@ -57,6 +67,15 @@ __device__ __forceinline__ double reciprocal(double x) {
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
 
+// sqrt(L) by one third-order step g (1 + e/2 + 3 e^2/8), g = L y, e = 1 - g y
+__device__ __forceinline__ double root(double L) {
+    const double y = rsqrt_seed(L);
+    const double g = __dmul_rn(L, y);
+    const double e = __fma_rn(-g, y, 1.0);
+    return __fma_rn(__dmul_rn(g, e), __fma_rn(e, 0.375, 0.5), g);
+}
+
+#ifndef FPT_NO_F64
 // -2 ln((w + 1/2) 2^-32)
 __device__ __forceinline__ double minus_two_ln(uint32_t w) {
     const uint64_t U = 2ull * w + 1ull;  // u0 = U 2^-33
@@ -70,14 +89,6 @@ __device__ __forceinline__ double minus_two_ln(uint32_t w) {
     q = __fma_rn(q, x, 1.0 / 12.0);
     q = __fma_rn(q, x, 0.25);
     return __dadd_rn(base, __fma_rn(__dmul_rn(x, x), q, x));
-}
-
-// sqrt(L) by one third-order step g (1 + e/2 + 3 e^2/8), g = L y, e = 1 - g y
-__device__ __forceinline__ double root(double L) {
-    const double y = rsqrt_seed(L);
-    const double g = __dmul_rn(L, y);
-    const double e = __fma_rn(-g, y, 1.0);
-    return __fma_rn(__dmul_rn(g, e), __fma_rn(e, 0.375, 0.5), g);
 }
 
 __device__ __forceinline__ PairF64 pair_f64(uint32_t rad, uint32_t h) {
@@ -101,5 +112,7 @@ __device__ __forceinline__ void normals4_f64(const PhiloxLane& l, uint32_t k, co
         xi[2 * p + 1] = __dmul_rn(q.r, q.s);
     }
 }
+
+#endif  // FPT_NO_F64
 
 }  // namespace fpt

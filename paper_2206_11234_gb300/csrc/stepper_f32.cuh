@@ -1,6 +1,7 @@
 // Binary32-state instantiations of the persistent stepper, for one of the two
 // log-weight sums per translation unit.
 #pragma once
+#define FPT_NO_F64
 #include "stepper.cuh"
 #include "stepper_few.cuh"
 #include "stepper_launch.h"

@@ -15,6 +15,7 @@
 #include <cstring>
 #include <vector>
 
+#define FPT_NO_F64
 #include "abi_internal.h"
 #include "fpt.h"
 #include "mlp.cuh"

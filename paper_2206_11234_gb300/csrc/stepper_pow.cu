@@ -1,6 +1,7 @@
 // Binary32-state instantiations of the persistent stepper with the power-law
 // bias B = A_p phi^p (§3.4 Eq. (26)): p in 0..4 specialised, any other real p
 // through exp2/log2; folds of 32 steps.
+#define FPT_NO_F64
 #include "stepper.cuh"
 #include "stepper_few.cuh"
 #include "stepper_launch.h"
